@@ -725,9 +725,11 @@ int enqueue_inner(const MixedState &S, cudaStream_t st, int *kernels) {
   return DTR_OK;
 }
 
+// Everything a captured graph holds by address or value.  Every link array is in it: a gauge field
+// freed and made again may get some of its old addresses back and others not.
 struct GraphKey {
   int device;
-  const void *U64, *U32;
+  const void *U64, *U32, *Udf;
   int L[4];
   double m0;
   const void *x, *z, *work;
@@ -893,6 +895,7 @@ static int solve_mixed_graph(const MixedState &S, int x_is_zero, double tol2, in
   DTR_CUDA(cudaGetDevice(&key.device));
   key.U64 = S.gauge->U64;
   key.U32 = S.gauge->U32;
+  key.Udf = S.gauge->Udf;
   for (int i = 0; i < 4; ++i) key.L[i] = S.g.L[i];
   key.m0 = S.m0;
   key.x = S.x;
