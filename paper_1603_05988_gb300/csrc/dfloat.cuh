@@ -15,7 +15,7 @@
 // the error-free transformations.
 #pragma once
 
-#include "dtr_internal.cuh"
+#include "dslash_core.cuh"
 
 namespace dtr {
 
@@ -111,9 +111,10 @@ __device__ __forceinline__ cdf cjmul(cdf a, cdf b) {
 __device__ __forceinline__ cdf caxpy(cdf s, cdf b, cdf a) { return cadd(a, cmul(s, b)); }
 
 // FP64 field value held as double-float hi + lo arrays (written by k_split_df)
-struct DfPairLoad {
+struct DfPairLoad : LexIndex {
   const float2 *__restrict__ hi;
   const float2 *__restrict__ lo;
+  __device__ __forceinline__ DfPairLoad(const float2 *h, const float2 *l) : hi(h), lo(l) {}
   __device__ __forceinline__ cdf operator()(int64_t idx) const {
     const float2 h = hi[idx], l = lo[idx];
     return mkc2(dff(h.x, l.x), dff(h.y, l.y));
@@ -121,8 +122,24 @@ struct DfPairLoad {
 };
 
 // FP32 field value as a df complex (exact)
-struct F32AsDf {
+struct F32AsDf : LexIndex {
   const float2 *__restrict__ f;
+  __device__ __forceinline__ explicit F32AsDf(const float2 *q) : f(q) {}
+  __device__ __forceinline__ cdf operator()(int64_t idx) const {
+    const float2 v = f[idx];
+    return mkc2(dff(v.x), dff(v.y));
+  }
+};
+// the same for a field in red-black order, [parity][site >> 1][12][bi]: the even sites first
+struct EoF32AsDf {
+  const float2 *__restrict__ f;
+  int64_t off_self, off_nbr;  // start of the site's own sublattice and of its neighbours'
+  int bi;
+  __device__ __forceinline__ EoF32AsDf(const float2 *q, int parity, int64_t half, int bi_)
+      : f(q), off_self(parity ? half : 0), off_nbr(parity ? 0 : half), bi(bi_) {}
+  __device__ __forceinline__ int64_t nbr(int s, int, int j) const { return off_nbr + (int64_t)(s >> 1) * 12 * bi + j; }
+  __device__ __forceinline__ int64_t self(int s, int, int j) const { return off_self + (int64_t)(s >> 1) * 12 * bi + j; }
+  __device__ __forceinline__ int stride(int) const { return bi; }
   __device__ __forceinline__ cdf operator()(int64_t idx) const {
     const float2 v = f[idx];
     return mkc2(dff(v.x), dff(v.y));

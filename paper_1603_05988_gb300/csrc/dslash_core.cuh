@@ -25,19 +25,18 @@
 
 namespace dtr {
 
-// Field loaders: value of the input field at internal index (site*12 + c)*b + j.
-template <typename C> struct PlainLoad {
+// Field loaders: value of the input field at an index; nbr/self give the index of component 0 of right-hand side j
+// at a neighbour or at the stencil's own site, stride the distance between components.
+struct LexIndex {  // whole-lattice fields [site][12][b]
+  __device__ __forceinline__ int64_t nbr(int s, int b, int j) const { return (int64_t)s * 12 * b + j; }
+  __device__ __forceinline__ int64_t self(int s, int b, int j) const { return (int64_t)s * 12 * b + j; }
+  __device__ __forceinline__ int stride(int b) const { return b; }
+};
+template <typename C> struct PlainLoad : LexIndex {
+  __device__ __forceinline__ explicit PlainLoad(const C *q) : f(q) {}
   const C *__restrict__ f;
   __device__ __forceinline__ C operator()(int64_t idx) const { return f[idx]; }
 };
-// s = r - a v evaluated on the fly (a is this thread's column scalar)
-template <typename C> struct AxpyLoad {
-  const C *__restrict__ r;
-  const C *__restrict__ v;
-  C a;
-  __device__ __forceinline__ C operator()(int64_t idx) const { return caxpy(cneg(a), v[idx], r[idx]); }
-};
-
 // Complex values stored as S, computed as float2/double2: loads widen, stores round to nearest.
 template <typename S> struct CStore {
   __device__ __forceinline__ static S ld(const S *p, int64_t i) { return p[i]; }
@@ -55,11 +54,14 @@ template <> struct CStore<__nv_bfloat162> {
     p[i] = __float22bfloat162_rn(v);
   }
 };
-template <typename S, typename C> struct PlainLoadS {
+template <typename S, typename C> struct PlainLoadS : LexIndex {
+  __device__ __forceinline__ explicit PlainLoadS(const S *q) : f(q) {}
   const S *__restrict__ f;
   __device__ __forceinline__ C operator()(int64_t idx) const { return CStore<S>::ld(f, idx); }
 };
-template <typename S, typename C> struct AxpyLoadS {
+// s = r - a v evaluated on the fly (a is this thread's column scalar)
+template <typename S, typename C> struct AxpyLoadS : LexIndex {
+  __device__ __forceinline__ AxpyLoadS(const S *r_, const S *v_, C a_) : r(r_), v(v_), a(a_) {}
   const S *__restrict__ r;
   const S *__restrict__ v;
   C a;
@@ -96,16 +98,17 @@ __device__ __forceinline__ void hop_dir(const typename cplx_t<R>::type *__restri
   const int sf = site_of(g, xf);
   const int sb = site_of(g, xb);
 
+  const int cs = in.stride(b);
   C wf[2][3], wb[2][3];
   {  // forward: h = u - sgn B l from psi(x+mu); w_f = U_mu(x) h
-    const int64_t p = (int64_t)sf * 12 * b + j;
+    const int64_t p = in.nbr(sf, b, j);
     C u[2][3], l[2][3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-      u[0][a] = in(p + (0 * 3 + a) * b);
-      u[1][a] = in(p + (1 * 3 + a) * b);
-      l[0][a] = in(p + (2 * 3 + a) * b);
-      l[1][a] = in(p + (3 * 3 + a) * b);
+      u[0][a] = in(p + (0 * 3 + a) * cs);
+      u[1][a] = in(p + (1 * 3 + a) * cs);
+      l[0][a] = in(p + (2 * 3 + a) * cs);
+      l[1][a] = in(p + (3 * 3 + a) * cs);
     }
     C h[2][3];
 #pragma unroll
@@ -133,14 +136,14 @@ __device__ __forceinline__ void hop_dir(const typename cplx_t<R>::type *__restri
       }
   }
   {  // backward: h' = u + sgn B l from psi(x-mu); w_b = U_mu(x-mu)^H h'
-    const int64_t p = (int64_t)sb * 12 * b + j;
+    const int64_t p = in.nbr(sb, b, j);
     C u[2][3], l[2][3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-      u[0][a] = in(p + (0 * 3 + a) * b);
-      u[1][a] = in(p + (1 * 3 + a) * b);
-      l[0][a] = in(p + (2 * 3 + a) * b);
-      l[1][a] = in(p + (3 * 3 + a) * b);
+      u[0][a] = in(p + (0 * 3 + a) * cs);
+      u[1][a] = in(p + (1 * 3 + a) * cs);
+      l[0][a] = in(p + (2 * 3 + a) * cs);
+      l[1][a] = in(p + (3 * 3 + a) * cs);
     }
     C h[2][3];
 #pragma unroll
@@ -207,9 +210,10 @@ __device__ __forceinline__ void dslash_site_ld(const typename cplx_t<R>::type *_
   hop_dir<1, SGN, R>(U, in, g, xc, s, b, j, Su, Sl);
   hop_dir<2, SGN, R>(U, in, g, xc, s, b, j, Su, Sl);
   hop_dir<3, SGN, R>(U, in, g, xc, s, b, j, Su, Sl);
-  const int64_t p = (int64_t)s * 12 * b + j;
+  const int64_t p = in.self(s, b, j);
+  const int cs = in.stride(b);
 #pragma unroll
-  for (int c = 0; c < 12; ++c) self[c] = in(p + c * b);
+  for (int c = 0; c < 12; ++c) self[c] = in(p + c * cs);
   const R half = (R)0.5;
 #pragma unroll
   for (int r = 0; r < 2; ++r)

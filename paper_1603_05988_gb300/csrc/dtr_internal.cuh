@@ -107,6 +107,12 @@ __device__ __forceinline__ int site_of(const Geom &g, const int c[4]) {
   return c[0] + g.L[0] * (c[1] + g.L[1] * (c[2] + g.L[2] * c[3]));
 }
 
+__device__ __forceinline__ int site_parity(const Geom &g, int s) {
+  int c[4];
+  site_coords(g, s, c);
+  return (c[0] + c[1] + c[2] + c[3]) & 1;
+}
+
 // Hierarchical-probing colour of a site; ncolors in {1, 2, 16, 32, 256, ...}.
 __host__ __device__ __forceinline__ int hp_colour(const int c[4], int ncolors) {
   if (ncolors <= 1) return 0;

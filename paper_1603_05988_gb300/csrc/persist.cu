@@ -33,6 +33,7 @@
 #include <vector>
 
 #include "dslash_core.cuh"
+#include "grid_barrier.cuh"
 #include "krylov_fin.cuh"
 #include <cstring>
 #include <type_traits>
@@ -41,50 +42,6 @@
 #include "reduce.cuh"
 
 namespace dtr {
-
-constexpr long long kSpinBudget = 4000000000LL;  // ~2 s at 2 GHz
-// Largest persistent grid: two buffers of 5 x 64 partials per block fit the
-// solver's reduction scratch (kMaxGrid x 5 x 64 double2).
-constexpr int kPersistMaxGrid = kMaxGrid / 2;
-
-__device__ __forceinline__ unsigned long long global_ns() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-
-// Counting grid barrier: arrive, then wait until `target` arrivals in total
-// (the barrier's sequence number times the grid size).  Returns false if the
-// wait exceeded `budget` clock cycles or another block reported an error.
-// Ordering without full fences: thread 0 arrives with a release reduction and
-// polls with acquire loads; the block barriers before and after extend that to
-// the whole block (the writes of the block's threads happen before the
-// release, and the acquire happens before their later reads).
-__device__ __forceinline__ bool grid_arrive_wait(GridSync *gs, unsigned int target, long long budget) {
-  __shared__ int s_err;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    s_err = 0;
-    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&gs->count) : "memory");
-    const long long t0 = clock64();
-    while (true) {
-      unsigned int c;
-      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(c) : "l"(&gs->count) : "memory");
-      if (c >= target) break;
-      if (*(volatile int *)&gs->error) {
-        s_err = 1;
-        break;
-      }
-      if (clock64() - t0 > budget) {
-        atomicExch(&gs->error, 1);
-        s_err = 1;
-        break;
-      }
-    }
-  }
-  __syncthreads();
-  return !s_err;
-}
 
 // Self-test: one block waits at a barrier that expects two arrivals, so the
 // peer never arrives and the bounded wait must give up with the error word set.
@@ -299,7 +256,7 @@ __global__ void __launch_bounds__(T, 1) k_bicgstab_persistent(PArgs<R, S> a) {
       if (blockIdx.x == 0 && threadIdx.x == 0) a.gs->iters = done;
       {  // P1: v = A p ; rhat^H v -> alpha   (per-thread sums in R, block/grid sums in FP64)
         R vx[1] = {0}, vy[1] = {0};
-        const PlainLoadS<S, C> ldp{a.p};
+        const PlainLoadS<S, C> ldp(a.p);
         for (int64_t it = t0; it < nsite; it += stride) {
           const int s = (int)(it >> logb);
           C o[12], self[12];
@@ -324,7 +281,7 @@ __global__ void __launch_bounds__(T, 1) k_bicgstab_persistent(PArgs<R, S> a) {
       int n_active = 0;
       {  // P2: t = A s with s = r - alpha v on the fly ; five dots -> omega, beta, convergence
         const C al = mkc<C>(ss.alpha[j]);
-        AxpyLoadS<S, C> ld{a.r, a.v, al};
+        AxpyLoadS<S, C> ld(a.r, a.v, al);
         R vx[5] = {0, 0, 0, 0, 0}, vy[5] = {0, 0, 0, 0, 0};
         for (int64_t it = t0; it < nsite; it += stride) {
           const int s = (int)(it >> logb);

@@ -21,6 +21,7 @@
 #include "reduce.cuh"
 #include "solver.cuh"
 #include "krylov_fin.cuh"
+#include "mixed_eo.cuh"
 #include "net.cuh"
 #include "persist.cuh"
 
@@ -125,6 +126,8 @@ __global__ void __launch_bounds__(kBlock) k_resid_zero(const double2 *__restrict
 // residual (k_resid_df) confirms convergence before the solve reports it.
 // (Two blocks per SM: the register cap spills ~500 B per thread to L1, yet the solve runs ~2% faster
 // than with one block of 255-register threads.)
+// EO: e is in red-black order, [parity][site >> 1][12][max(b, 2)].
+template <bool EO>
 __global__ void __launch_bounds__(kBlock, 2) k_resid_update(const cdf *__restrict__ Udf, const float2 *__restrict__ e,
                                                          double2 *__restrict__ r, Geom g, int b, int logb, dff diag,
                                                          double hs, Scal *sc, Reduce red, const int *run_flag,
@@ -135,13 +138,17 @@ __global__ void __launch_bounds__(kBlock, 2) k_resid_update(const cdf *__restric
   const int64_t n = (int64_t)g.V << logb;
   const int j = threadIdx.x & (b - 1);
   const double inv = sc->active[j] ? 1.0 / (sc->scale[j] * hs) : 0.0;
-  const F32AsDf ld{e};
+  const int bi = b < 2 ? 2 : b;
+  const int64_t half = (int64_t)(g.V >> 1) * 12 * bi;
   for (int64_t it = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; it < n; it += (int64_t)gridDim.x * blockDim.x) {
     const int s = (int)(it >> logb);
     const int64_t base = (int64_t)s * 12 * b + j;
     if (inv != 0.0) {
       cdf o[12], self[12];
-      dslash_site_ld<1, dff>(Udf, ld, g, b, s, j, diag, o, self);
+      if (EO)
+        dslash_site_ld<1, dff>(Udf, EoF32AsDf(e, site_parity(g, s), half, bi), g, b, s, j, diag, o, self);
+      else
+        dslash_site_ld<1, dff>(Udf, F32AsDf(e), g, b, s, j, diag, o, self);
 #pragma unroll
       for (int c = 0; c < 12; ++c) {
         double2 rr = r[base + c * b];
@@ -216,7 +223,7 @@ __global__ void __launch_bounds__(kBlock, 2) k_resid_df(const cdf *__restrict__ 
   double2 acc[1] = {make_double2(0.0, 0.0)};
   const int64_t n = (int64_t)g.V << logb;
   const int j = threadIdx.x & (b - 1);
-  const DfPairLoad ld{xhi, xlo};
+  const DfPairLoad ld(xhi, xlo);
   for (int64_t it = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; it < n; it += (int64_t)gridDim.x * blockDim.x) {
     const int s = (int)(it >> logb);
     const int64_t base = (int64_t)s * 12 * b + j;
@@ -282,7 +289,7 @@ __global__ void __launch_bounds__(kBlock) k_dslash_df(const cdf *__restrict__ Ud
                                                       double2 *__restrict__ out, Geom g, int b, int logb, dff diag) {
   const int64_t n = (int64_t)g.V << logb;
   const int j = threadIdx.x & (b - 1);
-  const F32AsDf ld{in};
+  const F32AsDf ld(in);
   for (int64_t it = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; it < n; it += (int64_t)gridDim.x * blockDim.x) {
     const int s = (int)(it >> logb);
     const int64_t base = (int64_t)s * 12 * b + j;
@@ -604,7 +611,10 @@ size_t solver_scratch_bytes(int64_t V, int b, int solver, int gmres_m) {
   const size_t red = 256 + (size_t)kMaxGrid * 5 * 64 * sizeof(double2);
   const size_t scal = 2 * ((sizeof(Scal) + 255) / 256) * 256;
   const size_t fixed = 256 + red + scal + 256 + 256;
-  if (mixed_bicgstab(solver)) return fixed + vec64 + 7 * vec32;  // half storage uses half of each slot
+  if (mixed_bicgstab(solver)) {  // half storage uses half of each slot; the larger of the two cycles' buffers
+    const size_t full = 7 * vec32, eo = eo_scratch_bytes(V, b);
+    return fixed + vec64 + (full > eo ? full : eo);
+  }
   if (solver == DTR_SOLVER_FGMRES_NET) return fixed + vec64 + 7 * vec32 + fgmres_scratch_bytes(V, b, gmres_m) + 256;
   return fixed + 6 * vec64;
 }
@@ -666,7 +676,31 @@ struct MixedState {
   int store;  // inner Krylov vectors: 0 FP32, 1 FP16, 2 BF16
   double hs;  // inner right-hand-side scale (see k_mixed_init)
   int upd;    // cycles end with the double-float residual update (then one true-residual verification)
+  int eo;     // inner solves on the red-black Schur complement (buffers B), else on the whole lattice (K, sv)
+  EoBufs B;
+  float2 *xhi, *xlo;  // x split for the true residual: idle between inner solves
 };
+
+// hands out the buffers of the mixed solvers' cycles from the workspace after the fixed part
+static void carve_mixed(MixedState &S, char *w) {
+  const int64_t n = (int64_t)S.g.V * 12 * S.b;
+  S.r64 = (double2 *)w; w = align256(w + n * sizeof(double2));
+  if (S.eo) {
+    S.B = eo_carve(w, S.g.V, S.b);
+    S.xhi = (float2 *)S.B.r;          // six half-lattice fields from here on
+    S.xlo = S.xhi + n;
+    return;
+  }
+  S.K.x = (float2 *)w;    w = align256(w + n * sizeof(float2));
+  S.K.r = (float2 *)w;    w = align256(w + n * sizeof(float2));
+  S.K.rhat = (float2 *)w; w = align256(w + n * sizeof(float2));
+  S.K.p = (float2 *)w;    w = align256(w + n * sizeof(float2));
+  S.K.v = (float2 *)w;    w = align256(w + n * sizeof(float2));
+  S.K.t = (float2 *)w;    w = align256(w + n * sizeof(float2));
+  S.sv = (float2 *)w;
+  S.xhi = S.K.v;
+  S.xlo = S.K.t;
+}
 
 // inner iterations of one defect-correction cycle on the caller-initialised state
 template <typename S>
@@ -710,8 +744,14 @@ static int inner_solve(int store, const dtr_gauge_s *gauge, const KrylovVecs<flo
   return launch_inner<float2>(gauge, K, sv, g, b, logb, m0, inner, red, gs, maxiter, grid, st);
 }
 
-// One defect-correction cycle after a residual: returns the kernels it launched.
+// Inner solve of one defect-correction cycle after a residual (persistent engine); kernels: those it launched.
 int enqueue_inner(const MixedState &S, cudaStream_t st, int *kernels) {
+  if (S.eo) {
+    const int rc = eo_inner(S.gauge, S.B, S.g, S.b, S.m0, S.r64, S.outer, S.inner, S.red, S.gs, S.itol * S.itol,
+                            S.maxiter, S.hs, S.store, S.grid, st, kernels);
+    *kernels += persist_profile().on ? 1 : 0;
+    return rc;
+  }
   const int64_t n = (int64_t)S.g.V * 12 * S.b;
   mixed_init(S.store, S.r64, S.K, n, S.b, S.outer, S.hs, S.gv, st);
   k_mixed_scal_init<<<1, 64, 0, st>>>(S.outer, S.inner, S.b, S.itol * S.itol, S.maxiter, S.hs * S.hs);
@@ -725,6 +765,37 @@ int enqueue_inner(const MixedState &S, cudaStream_t st, int *kernels) {
   return DTR_OK;
 }
 
+// x += the cycle's correction, choosing the next residual if choose (one kernel)
+void enqueue_accum(const MixedState &S, int choose, cudaStream_t st) {
+  if (S.eo) {
+    eo_accum(S.gauge, S.B, S.g, S.b, S.m0, S.x, S.outer, S.inner, S.hs, choose ? S.gs : nullptr, choose, st);
+    return;
+  }
+  k_mixed_accum<<<S.gv, kBlock, 0, st>>>(S.x, S.K.x, (int64_t)S.g.V * 12 * S.b, S.b, S.outer, S.inner, S.hs,
+                                         choose ? S.gs : nullptr, choose);
+  count_launches(1);
+}
+
+// the double-float residual update, run if gs->sel is 1 (one kernel)
+void enqueue_resid_update(const MixedState &S, cudaStream_t st) {
+  const cdf *U = (const cdf *)S.gauge->Udf;
+  const dff d = split_df(4.0 + S.m0);
+  if (S.eo)
+    k_resid_update<true><<<S.gd, kBlock, 0, st>>>(U, S.B.e, S.r64, S.g, S.b, S.logb, d, S.hs, S.outer, S.red,
+                                                  &S.gs->sel, 1, &S.gs->last_upd);
+  else
+    k_resid_update<false><<<S.gd, kBlock, 0, st>>>(U, S.K.x, S.r64, S.g, S.b, S.logb, d, S.hs, S.outer, S.red,
+                                                   &S.gs->sel, 1, &S.gs->last_upd);
+  count_launches(1);
+}
+
+// the true residual (three kernels), run if *run_flag == run_if (NULL: always)
+void enqueue_true_resid(const MixedState &S, int restart, const int *run_flag, int run_if, cudaStream_t st) {
+  launch_true_resid_df(S.gauge, S.x, S.z, S.r64, S.xhi, S.xlo, S.g, S.b, S.logb, S.m0, S.outer, S.red, restart,
+                       run_flag, run_if, &S.gs->last_upd, &S.gs->fp64_cert, S.gd, S.gv, st);
+  count_launches(3);
+}
+
 // Everything a captured graph holds by address or value.  Every link array is in it: a gauge field
 // freed and made again may get some of its old addresses back and others not.
 struct GraphKey {
@@ -733,7 +804,7 @@ struct GraphKey {
   int L[4];
   double m0;
   const void *x, *z, *work;
-  int b, x_is_zero, maxiter, grid, prof, store, upd, pad2;
+  int b, x_is_zero, maxiter, grid, prof, store, upd, eo;
   double tol, itol;
 };
 
@@ -795,8 +866,7 @@ int capture_mixed_graph(const MixedState &S, int x_is_zero, double tol2, int max
   if (x_is_zero)
     k_resid_zero<<<S.gv, kBlock, 0, cs>>>(S.z, S.r64, n, S.b, S.outer, S.red);
   else
-    launch_true_resid_df(S.gauge, S.x, S.z, S.r64, S.K.v, S.K.t, S.g, S.b, S.logb, S.m0, S.outer, S.red, 1, nullptr,
-                         0, &S.gs->last_upd, &S.gs->fp64_cert, S.gd, S.gv, cs);
+    enqueue_true_resid(S, 1, nullptr, 0, cs);
   unsigned long long *devcnt = device_launch_counter();
   k_loop_cond<<<1, 32, 0, cs>>>(h, S.outer, S.gs, (unsigned)kMaxRestarts + 1, 1, devcnt, 0);
   CAP_CHECK(cudaGetLastError());
@@ -818,13 +888,9 @@ int capture_mixed_graph(const MixedState &S, int x_is_zero, double tol2, int max
   int kin = 0;
   rc = enqueue_inner(S, cs2, &kin);
   if (rc) return bail(rc);
-  k_mixed_accum<<<S.gv, kBlock, 0, cs2>>>(S.x, S.K.x, n, S.b, S.outer, S.inner, S.hs, S.gs, S.upd);
-  if (S.upd)  // one of the two runs, as k_mixed_accum chose
-    k_resid_update<<<S.gd, kBlock, 0, cs2>>>((const cdf *)S.gauge->Udf, S.K.x, S.r64, S.g, S.b, S.logb,
-                                             split_df(4.0 + S.m0), S.hs, S.outer, S.red, &S.gs->sel, 1,
-                                             &S.gs->last_upd);
-  launch_true_resid_df(S.gauge, S.x, S.z, S.r64, S.K.v, S.K.t, S.g, S.b, S.logb, S.m0, S.outer, S.red, 1,
-                       S.upd ? &S.gs->sel : nullptr, 0, &S.gs->last_upd, &S.gs->fp64_cert, S.gd, S.gv, cs2);
+  enqueue_accum(S, S.upd, cs2);
+  if (S.upd) enqueue_resid_update(S, cs2);  // one of the two runs, as the accumulation chose
+  enqueue_true_resid(S, 1, S.upd ? &S.gs->sel : nullptr, 0, cs2);
   k_loop_cond<<<1, 32, 0, cs2>>>(h, S.outer, S.gs, (unsigned)kMaxRestarts + 1, 0, devcnt,
                                  (unsigned)(kin + (S.upd ? 6 : 5)));
   CAP_CHECK(cudaGetLastError());
@@ -835,8 +901,7 @@ int capture_mixed_graph(const MixedState &S, int x_is_zero, double tol2, int max
     // verification (when the loop ended on a double-float update): the true residual
     // of x decides; columns it finds short of tol continue in a second loop whose
     // cycles end with the true residual
-    launch_true_resid_df(S.gauge, S.x, S.z, S.r64, S.K.v, S.K.t, S.g, S.b, S.logb, S.m0, S.outer, S.red, 1,
-                         &S.gs->last_upd, 1, &S.gs->last_upd, &S.gs->fp64_cert, S.gd, S.gv, cs);
+    enqueue_true_resid(S, 1, &S.gs->last_upd, 1, cs);
     cudaGraphConditionalHandle h2;
     CAP_CHECK(cudaGraphConditionalHandleCreate(&h2, graph, 0, 0));
     k_loop_cond<<<1, 32, 0, cs>>>(h2, S.outer, S.gs, (unsigned)kMaxRestarts + 1, 2, devcnt, 0);
@@ -854,9 +919,8 @@ int capture_mixed_graph(const MixedState &S, int x_is_zero, double tol2, int max
     open = 2;
     rc = enqueue_inner(S, cs2, &kin);
     if (rc) return bail(rc);
-    k_mixed_accum<<<S.gv, kBlock, 0, cs2>>>(S.x, S.K.x, n, S.b, S.outer, S.inner, S.hs, nullptr, 0);
-    launch_true_resid_df(S.gauge, S.x, S.z, S.r64, S.K.v, S.K.t, S.g, S.b, S.logb, S.m0, S.outer, S.red, 1, nullptr,
-                         0, &S.gs->last_upd, &S.gs->fp64_cert, S.gd, S.gv, cs2);
+    enqueue_accum(S, 0, cs2);
+    enqueue_true_resid(S, 1, nullptr, 0, cs2);
     k_loop_cond<<<1, 32, 0, cs2>>>(h2, S.outer, S.gs, (unsigned)kMaxRestarts + 1, 0, devcnt, (unsigned)(kin + 5));
     CAP_CHECK(cudaGetLastError());
     CAP_CHECK(cudaStreamEndCapture(cs2, &tmp));
@@ -910,6 +974,7 @@ static int solve_mixed_graph(const MixedState &S, int x_is_zero, double tol2, in
   key.itol = S.itol;
   key.store = S.store;
   key.upd = S.upd;
+  key.eo = S.eo;
   std::lock_guard<std::mutex> lock(g_graph_mu);
   GraphEntry *hit = nullptr;
   for (auto &e : g_graphs)
@@ -992,24 +1057,18 @@ int solve_internal(const dtr_gauge_s *gauge, double m0, double2 *x, const double
   const double hs = store ? std::sqrt(12.0 * (double)g.V) : 1.0;
   const double itol = inner_tol_for(p);
   if (store && !persistent) return fail(DTR_EINVAL, "half-storage inner solves need the persistent engine");
+  MixedState S;  // the mixed solvers' and FGMRES' outer loop
+  S.gauge = gauge; S.g = g; S.b = b; S.logb = logb; S.m0 = m0; S.x = x; S.z = z;
+  S.outer = outer; S.inner = inner; S.red = red; S.gs = gs; S.gd = gd; S.gv = gv;
+  S.itol = itol;
+  S.maxiter = p->maxiter;
+  S.grid = p->grid;
+  S.store = store;
+  S.hs = hs;
+  S.upd = resid_update_enabled(store) ? 1 : 0;
+  S.eo = mixed_bicgstab(p->solver) && persistent && eo_usable(m0);
   if (mixed_bicgstab(p->solver) && persistent && !p->no_graph) {
-    MixedState S;
-    S.gauge = gauge; S.g = g; S.b = b; S.logb = logb; S.m0 = m0; S.x = x; S.z = z;
-    S.r64 = (double2 *)w; w = align256(w + n * sizeof(double2));
-    S.K.x = (float2 *)w;    w = align256(w + n * sizeof(float2));
-    S.K.r = (float2 *)w;    w = align256(w + n * sizeof(float2));
-    S.K.rhat = (float2 *)w; w = align256(w + n * sizeof(float2));
-    S.K.p = (float2 *)w;    w = align256(w + n * sizeof(float2));
-    S.K.v = (float2 *)w;    w = align256(w + n * sizeof(float2));
-    S.K.t = (float2 *)w;    w = align256(w + n * sizeof(float2));
-    S.sv = (float2 *)w;     w = align256(w + n * sizeof(float2));
-    S.outer = outer; S.inner = inner; S.red = red; S.gs = gs; S.gd = gd; S.gv = gv;
-    S.itol = itol;
-    S.maxiter = p->maxiter;
-    S.grid = p->grid;
-    S.store = store;
-    S.hs = hs;
-    S.upd = resid_update_enabled(store) ? 1 : 0;
+    carve_mixed(S, w);
     *scal_out = outer;
     int rc = solve_mixed_graph(S, x_is_zero, p->tol * p->tol, p->maxiter, work, st);
     if (rc) return rc;
@@ -1056,16 +1115,9 @@ int solve_internal(const dtr_gauge_s *gauge, double m0, double2 *x, const double
     return DTR_OK;
   }
   if (mixed_bicgstab(p->solver) || p->solver == DTR_SOLVER_FGMRES_NET) {
-    double2 *r64 = (double2 *)w; w = align256(w + n * sizeof(double2));
-    KrylovVecs<float> K;
-    K.x = (float2 *)w;    w = align256(w + n * sizeof(float2));
-    K.r = (float2 *)w;    w = align256(w + n * sizeof(float2));
-    K.rhat = (float2 *)w; w = align256(w + n * sizeof(float2));
-    K.p = (float2 *)w;    w = align256(w + n * sizeof(float2));
-    K.v = (float2 *)w;    w = align256(w + n * sizeof(float2));
-    K.t = (float2 *)w;    w = align256(w + n * sizeof(float2));
-    float2 *sv = (float2 *)w; w = align256(w + n * sizeof(float2));
-    void *fg_work = w;
+    carve_mixed(S, w);
+    KrylovVecs<float> &K = S.K;
+    void *fg_work = S.eo ? nullptr : align256((char *)(S.sv + n));
     const size_t fg_bytes = p->solver == DTR_SOLVER_FGMRES_NET ? fgmres_scratch_bytes(g.V, b, p->gmres_m) : 0;
     bool fgmres = p->solver == DTR_SOLVER_FGMRES_NET;
     std::vector<double> prev_rel(64, -1.0);
@@ -1078,34 +1130,35 @@ int solve_internal(const dtr_gauge_s *gauge, double m0, double2 *x, const double
     for (int cycle = 0; cycle <= kMaxRestarts; ++cycle) {
       const int restart = cycle < kMaxRestarts;
       if (cycle == 0 && x_is_zero) {
-        k_resid_zero<<<gv, kBlock, 0, st>>>(z, r64, n, b, outer, red);
+        k_resid_zero<<<gv, kBlock, 0, st>>>(z, S.r64, n, b, outer, red);
         count_launches(1);
       } else if (cycle > 0 && upd_phase) {
-        k_resid_update<<<gd, kBlock, 0, st>>>((const cdf *)gauge->Udf, K.x, r64, g, b, logb, split_df(4.0 + m0), hs,
-                                              outer, red, &gs->sel, 1, &gs->last_upd);
-        launch_true_resid_df(gauge, x, z, r64, K.v, K.t, g, b, logb, m0, outer, red, restart, &gs->sel, 0,
-                             &gs->last_upd, &gs->fp64_cert, gd, gv, st);
-        count_launches(4);
+        enqueue_resid_update(S, st);
+        enqueue_true_resid(S, restart, &gs->sel, 0, st);
       } else {
-        launch_true_resid_df(gauge, x, z, r64, K.v, K.t, g, b, logb, m0, outer, red, restart, nullptr, 0,
-                             &gs->last_upd, &gs->fp64_cert, gd, gv, st);
-        count_launches(3);
+        enqueue_true_resid(S, restart, nullptr, 0, st);
       }
       DTR_LAUNCH_CHECK("outer residual");
       int n_active = 0;
       int rc = read_n_active(outer, st, &n_active);
       if (rc) return rc;
       if (n_active == 0 && cycle > 0 && upd_phase) {  // verify if the last residual was the update
-        launch_true_resid_df(gauge, x, z, r64, K.v, K.t, g, b, logb, m0, outer, red, restart, &gs->last_upd, 1,
-                             &gs->last_upd, &gs->fp64_cert, gd, gv, st);
-        count_launches(3);
+        enqueue_true_resid(S, restart, &gs->last_upd, 1, st);
         DTR_LAUNCH_CHECK("verification residual");
         upd_phase = false;
         rc = read_n_active(outer, st, &n_active);
         if (rc) return rc;
       }
       if (n_active == 0) break;
-      mixed_init(store, r64, K, n, b, outer, hs, gv, st);
+      if (mixed_bicgstab(p->solver) && persistent) {
+        int kernels = 0;
+        rc = enqueue_inner(S, st, &kernels);
+        if (rc) return rc;
+        enqueue_accum(S, upd_phase, st);
+        DTR_LAUNCH_CHECK("defect accumulate");
+        continue;
+      }
+      mixed_init(store, S.r64, K, n, b, outer, hs, gv, st);
       k_mixed_scal_init<<<1, 64, 0, st>>>(outer, inner, b, itol * itol, p->maxiter, hs * hs); count_launches(1);
       DTR_LAUNCH_CHECK("inner init");
       if (fgmres) {
@@ -1134,14 +1187,13 @@ int solve_internal(const dtr_gauge_s *gauge, double m0, double2 *x, const double
         DTR_CUDA(cudaMemcpyAsync(inner->iters, its.data(), sizeof(int) * b, cudaMemcpyHostToDevice, st));
       } else if (persistent) {
         DTR_CUDA(cudaMemsetAsync(gs, 0, kGridSyncLaunchBytes, st));
-        rc = inner_solve(store, gauge, K, sv, g, b, logb, m0, inner, red, gs, p->maxiter, p->grid, st);
+        rc = inner_solve(store, gauge, K, S.sv, g, b, logb, m0, inner, red, gs, p->maxiter, p->grid, st);
         if (rc) return rc;
       } else {
         rc = iterate<float>(gauge->U32, K, g, b, m0, inner, red, check, p->maxiter + check, st);
         if (rc) return rc;
       }
-      k_mixed_accum<<<gv, kBlock, 0, st>>>(x, K.x, n, b, outer, inner, hs, upd_phase ? gs : nullptr, upd_phase ? 1 : 0);
-      count_launches(1);
+      enqueue_accum(S, upd_phase, st);
       DTR_LAUNCH_CHECK("defect accumulate");
     }
     if (persistent) return read_gs_error(gs, st);
