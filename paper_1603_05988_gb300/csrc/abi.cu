@@ -76,6 +76,17 @@ __global__ void k_to_f32(const double2 *__restrict__ a, float2 *__restrict__ b, 
     b[i] = make_float2((float)a[i].x, (float)a[i].y);
 }
 
+// FP32 copies of n / 9 links, each padded to kLink32 entries
+__global__ void k_links_f32(const double2 *__restrict__ a, float2 *__restrict__ b, int64_t n) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t l = i / 9;
+    const int k = (int)(i - 9 * l);
+    const double2 v = a[i];
+    float2 *q = b + l * kLink32 + k;
+    q[0] = make_float2((float)v.x, (float)v.y);
+    if (k == 8) q[1] = make_float2(0.f, 0.f);
+  }
+}
 static unsigned grid1d(int64_t n) {
   int64_t g = (n + 255) / 256;
   if (g > 65535LL * 8) g = 65535LL * 8;
@@ -205,7 +216,7 @@ static int gauge_create(dtr_lattice lat, const double *links_host, double eps, u
   g->Udf = nullptr;
   const int64_t n = lat->V * 4 * 9;
   cudaError_t e = cudaMalloc((void **)&g->U64, n * sizeof(double2));
-  if (e == cudaSuccess) e = cudaMalloc((void **)&g->U32, n * sizeof(float2));
+  if (e == cudaSuccess) e = cudaMalloc((void **)&g->U32, lat->V * 4 * kLink32 * sizeof(float2));
   if (e == cudaSuccess) e = cudaMalloc(&g->Udf, n * sizeof(float4));
   if (e == cudaSuccess) e = cudaMalloc(&g->Ubf16, half_links_bytes(lat->V));
   if (e == cudaSuccess) e = cudaMalloc(&g->Uf16, half_links_bytes(lat->V));
@@ -218,7 +229,7 @@ static int gauge_create(dtr_lattice lat, const double *links_host, double eps, u
     }
   }
   if (e == cudaSuccess) {
-    k_to_f32<<<grid1d(n), 256>>>(g->U64, g->U32, n); count_launches(1);
+    k_links_f32<<<grid1d(n), 256>>>(g->U64, g->U32, n); count_launches(1);
     k_split_links<<<grid1d(n), 256>>>(g->U64, (float4 *)g->Udf, n); count_launches(1);
     launch_pack_links_half(g->U64, g->Ubf16, lat->V, 1, 0);
     launch_pack_links_half(g->U64, g->Uf16, lat->V, 0, 0);

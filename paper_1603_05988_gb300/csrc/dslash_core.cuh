@@ -119,7 +119,7 @@ __device__ __forceinline__ void hop_dir(const typename cplx_t<R>::type *__restri
         h[r][a] = SGN > 0 ? csub(u[r][a], bl) : cadd(u[r][a], bl);
       }
     }
-    const C *Ul = U + ((int64_t)s * 4 + MU) * 9;
+    const C *Ul = U + ((int64_t)s * 4 + MU) * LinkStride<C>::value;
     C m[3][3];
 #pragma unroll
     for (int a = 0; a < 3; ++a)
@@ -154,7 +154,7 @@ __device__ __forceinline__ void hop_dir(const typename cplx_t<R>::type *__restri
         h[r][a] = SGN > 0 ? cadd(u[r][a], bl) : csub(u[r][a], bl);
       }
     }
-    const C *Ul = U + ((int64_t)sb * 4 + MU) * 9;
+    const C *Ul = U + ((int64_t)sb * 4 + MU) * LinkStride<C>::value;
     C m[3][3];
 #pragma unroll
     for (int a = 0; a < 3; ++a)

@@ -130,6 +130,12 @@ __host__ __device__ __forceinline__ int hp_colour(const int c[4], int ncolors) {
   return col;
 }
 
+// Complex entries from one stored link to the next: an FP32 link is padded to 80 bytes so that every link starts on
+// 16 bytes and takes five loads instead of nine (the stencils' load pipe is as busy with links as with fields).
+constexpr int kLink32 = 10;
+template <typename C> struct LinkStride { static constexpr int value = 9; };
+template <> struct LinkStride<float2> { static constexpr int value = kLink32; };
+
 // ------------------------------------------------------------------ handles
 }  // namespace dtr
 
@@ -142,7 +148,7 @@ struct dtr_lattice_s {
 struct dtr_gauge_s {
   dtr_lattice_s lat;
   double2 *U64;   // [site][mu][3][3], FP64
-  float2 *U32;    // same layout, FP32
+  float2 *U32;    // [site][mu][kLink32], FP32: nine entries and one of padding
   void *Ubf16;    // BF16 links of the half-precision stencil, AoSoA over sites: three stored rows
                   // (36 complex per site) or two (24), see half_link_rows()
   void *Uf16;     // same, FP16

@@ -14,9 +14,13 @@
 // sublattices are indexed by h = site >> 1, and the neighbours in y, z, t of the site at h lie at the same h
 // offsets as on the whole lattice.
 //
-// Fields are [h][12][b] complex (b a power of two, 2..64).  A thread works on columns 2 jp and 2 jp + 1 in the two
-// lanes of packed FP32x2 instructions (half the issue slots of the scalar form).  Krylov vectors are stored as
-// {Re_2jp, Re_2jp+1, Im_2jp, Im_2jp+1} so that a load lands in the lanes without moves.
+// Fields are [h][12][b] complex (b a power of two, 2..64).  A work item is one site, one column pair 2 jp, 2 jp + 1
+// and one spin row r (0 or 1): the columns sit in the two lanes of packed FP32x2 instructions (half the issue slots
+// of the scalar form), and the two threads of a site and pair (lanes of one warp) each do one row of the half spinors.
+// A row needs 6 of a neighbour's 12 components, none of them twice, so the split costs no field loads; it halves a
+// thread's registers, which buys the warps that hide the load latency, and doubles the threads of a small lattice.
+// Only the lower-spin sums of the x and y hops cross rows: they are exchanged once per site by shuffles.
+// Krylov vectors are stored as {Re_2jp, Re_2jp+1, Im_2jp, Im_2jp+1} so that a load lands in the lanes without moves.
 #pragma once
 
 #include <cuda_bf16.h>
@@ -42,12 +46,12 @@ __device__ __forceinline__ c2 axpy2(const s2 &s, c2 b, c2 a) {
   return c2{__ffma2_rn(s.re, b.re, __ffma2_rn(s.nim, b.im, a.re)),
             __ffma2_rn(s.re, b.im, __ffma2_rn(s.im, b.re, a.im))};
 }
-// u + w l for w = 1, i, -1, -i (W = 0..3)
-template <int W> __device__ __forceinline__ c2 addw(c2 u, c2 l) {
-  if (W == 0) return c2{__fadd2_rn(u.re, l.re), __fadd2_rn(u.im, l.im)};
-  if (W == 1) return c2{sub2(u.re, l.im), __fadd2_rn(u.im, l.re)};
-  if (W == 2) return c2{sub2(u.re, l.re), sub2(u.im, l.im)};
-  return c2{__fadd2_rn(u.re, l.im), sub2(u.im, l.re)};
+// u + s l and u + i s l, s real (+-1), n = -s
+__device__ __forceinline__ c2 adds(c2 u, c2 l, float2 s) {
+  return c2{__ffma2_rn(s, l.re, u.re), __ffma2_rn(s, l.im, u.im)};
+}
+__device__ __forceinline__ c2 addi(c2 u, c2 l, float2 s, float2 n) {
+  return c2{__ffma2_rn(n, l.im, u.re), __ffma2_rn(s, l.re, u.im)};
 }
 
 // ---------------------------------------------------------------- storage
@@ -75,102 +79,163 @@ template <> struct Pair2<__nv_bfloat16> {
   }
 };
 
-// Loaders: value of component c at half-lattice site h (columns 2 jp, 2 jp + 1); P = b / 2.
+// What a thread keeps for its work items: column pair, spin row and the offsets of its 6 components.  ROWBIT: the
+// bit of the thread index that is the spin row.  4 (a half warp per row) for fields of 16 bytes per pair, whose loads
+// go by quarter warps; 0 for the 8-byte ones (16^3 x 32 x 32, hop of A in us: FP32 140 against 148 with bit 0, FP16
+// 129 against 136 with bit 4).
+template <int ROWBIT> struct EoLane {
+  int P;                    // column pairs, b / 2
+  int jp;                   // this thread's
+  int r;                    // spin row
+  float2 sg, ng;            // +1, -1 for row 0; -1, +1 for row 1
+  int cu, clx, clz;         // components: u_r, and l of the row's partner in x, y (1 - r) and z, t (r), times P
+  __device__ __forceinline__ EoLane(int b, int tid) : P(b >> 1) {
+    r = (tid >> ROWBIT) & 1;
+    jp = (int)pair_of_item(tid) & (P - 1);
+    sg = f2(r ? -1.f : 1.f);
+    ng = f2(r ? 1.f : -1.f);
+    cu = 3 * r * P;
+    clx = (9 - 3 * r) * P;
+    clz = (6 + 3 * r) * P;
+  }
+  // (site, column pair) that thread item `it` works on: 16 of them a warp
+  __host__ __device__ __forceinline__ static constexpr int64_t pair_of_item(int64_t it) {
+    return ROWBIT ? (it >> 5) * 16 + (it & 15) : it >> 1;
+  }
+  // v of the thread with the other spin row
+  __device__ __forceinline__ static float2 other_row(float2 v) {
+    return make_float2(__shfl_xor_sync(0xffffffffu, v.x, 1 << ROWBIT), __shfl_xor_sync(0xffffffffu, v.y, 1 << ROWBIT));
+  }
+};
+template <typename S> constexpr int row_bit() { return sizeof(typename Pair2<S>::T) == 16 ? 4 : 0; }
+
+// Loaders: load(h, cl) fetches components c + a P (a = 0, 1, 2) of u and l at half-lattice site h, value() turns them
+// into FP32 pairs (apart, so that the next hop's loads are in flight while this one is computed).
 template <typename S> struct PairLoad {
-  const typename Pair2<S>::T *f;
-  int P, jp;
-  __device__ __forceinline__ void get(int h, const int (&c)[12], c2 (&o)[12]) const {
-    const typename Pair2<S>::T *q = f + (int64_t)h * 12 * P + jp;
-    typename Pair2<S>::T v[12];
+  typedef typename Pair2<S>::T ST;
+  struct Raw {
+    ST u[3], l[3];
+  };
+  const ST *f;
+  template <class LN> __device__ __forceinline__ Raw load(const LN &ln, int h, int cl) const {
+    const ST *q = f + (int64_t)h * 12 * ln.P + ln.jp;
+    Raw w;
 #pragma unroll
-    for (int k = 0; k < 12; ++k) v[k] = q[c[k]];
+    for (int k = 0; k < 3; ++k) {
+      w.u[k] = q[ln.cu + k * ln.P];
+      w.l[k] = q[cl + k * ln.P];
+    }
+    return w;
+  }
+  __device__ __forceinline__ void value(const Raw &w, c2 (&u)[3], c2 (&l)[3]) const {
 #pragma unroll
-    for (int k = 0; k < 12; ++k) o[k] = Pair2<S>::widen(v[k]);
+    for (int k = 0; k < 3; ++k) {
+      u[k] = Pair2<S>::widen(w.u[k]);
+      l[k] = Pair2<S>::widen(w.l[k]);
+    }
   }
 };
 // r - a v on the fly
 template <typename S> struct PairAxpyLoad {
-  const typename Pair2<S>::T *r;
-  const typename Pair2<S>::T *v;
-  int P, jp;
+  typedef typename Pair2<S>::T ST;
+  struct Raw {
+    typename PairLoad<S>::Raw r, v;
+  };
+  const ST *r;
+  const ST *v;
   s2 ma;  // -a
-  __device__ __forceinline__ void get(int h, const int (&c)[12], c2 (&o)[12]) const {
-    const int64_t q = (int64_t)h * 12 * P + jp;
-    typename Pair2<S>::T rr[12], vv[12];
+  template <class LN> __device__ __forceinline__ Raw load(const LN &ln, int h, int cl) const {
+    return Raw{PairLoad<S>{r}.load(ln, h, cl), PairLoad<S>{v}.load(ln, h, cl)};
+  }
+  __device__ __forceinline__ void value(const Raw &w, c2 (&u)[3], c2 (&l)[3]) const {
 #pragma unroll
-    for (int k = 0; k < 12; ++k) {
-      rr[k] = r[q + c[k]];
-      vv[k] = v[q + c[k]];
+    for (int k = 0; k < 3; ++k) {
+      u[k] = axpy2(ma, Pair2<S>::widen(w.v.u[k]), Pair2<S>::widen(w.r.u[k]));
+      l[k] = axpy2(ma, Pair2<S>::widen(w.v.l[k]), Pair2<S>::widen(w.r.l[k]));
     }
-#pragma unroll
-    for (int k = 0; k < 12; ++k) o[k] = axpy2(ma, Pair2<S>::widen(vv[k]), Pair2<S>::widen(rr[k]));
   }
 };
 // FP32 field stored as interleaved complex columns, [h][12][b] float2
+__device__ __forceinline__ c2 from_cols(float4 v) { return c2{make_float2(v.x, v.z), make_float2(v.y, v.w)}; }
+__device__ __forceinline__ float4 to_cols(c2 v) { return make_float4(v.re.x, v.im.x, v.re.y, v.im.y); }
 struct CplxLoad {
-  const float2 *__restrict__ f;
-  int P, jp;
-  __device__ __forceinline__ void get(int h, const int (&c)[12], c2 (&o)[12]) const {
-    const float4 *q = (const float4 *)f + (int64_t)h * 12 * P + jp;
-    float4 v[12];
+  struct Raw {
+    float4 u[3], l[3];
+  };
+  const float2 *f;
+  template <class LN> __device__ __forceinline__ Raw load(const LN &ln, int h, int cl) const {
+    const float4 *q = (const float4 *)f + (int64_t)h * 12 * ln.P + ln.jp;
+    Raw w;
 #pragma unroll
-    for (int k = 0; k < 12; ++k) v[k] = q[c[k]];
+    for (int k = 0; k < 3; ++k) {
+      w.u[k] = q[ln.cu + k * ln.P];
+      w.l[k] = q[cl + k * ln.P];
+    }
+    return w;
+  }
+  __device__ __forceinline__ void value(const Raw &w, c2 (&u)[3], c2 (&l)[3]) const {
 #pragma unroll
-    for (int k = 0; k < 12; ++k) o[k] = c2{make_float2(v[k].x, v[k].z), make_float2(v[k].y, v[k].w)};
+    for (int k = 0; k < 3; ++k) {
+      u[k] = from_cols(w.u[k]);
+      l[k] = from_cols(w.l[k]);
+    }
+  }
+  template <class LN> __device__ __forceinline__ void get(const LN &ln, int h, int cl, c2 (&u)[3], c2 (&l)[3]) const {
+    value(load(ln, h, cl), u, l);
   }
 };
 
 // ---------------------------------------------------------------- stencil
-// Su += w, Sl += +-B^H w for w = U h (FWD) or U^H h, h = u -+ B l the half spinor of the neighbour at hn.
-template <int MU, bool FWD, class LD>
-__device__ __forceinline__ void hop_eo_dir(const float2 *__restrict__ Ul, const LD &in, int hn, const int (&c)[12],
-                                           c2 (&Su)[2][3], c2 (&Sl)[2][3]) {
-  c2 f[12];
-  in.get(hn, c, f);
+// One hop for one spin row: Su += w, L += +-B^H w, w = U h (FWD) or U^H h, h = u - B l (FWD) or u + B l the row of
+// the neighbour's half spinor (raw: its loaded components).
+template <int MU, bool FWD, class LN, class LD>
+__device__ __forceinline__ void hop_eo_dir(const LN &ln, const float2 *__restrict__ Ul, const LD &in,
+                                           const typename LD::Raw &raw, c2 (&Su)[3], c2 (&L)[3]) {
+  c2 h[3], l[3];
+  in.value(raw, h, l);
   float2 m[9];
+  {
+    const float4 *q = (const float4 *)Ul;
 #pragma unroll
-  for (int k = 0; k < 9; ++k) m[k] = __ldg(Ul + k);
-  // B l = (-i l1, -i l0), (-l1, l0), (-i l0, i l1), (l0, l1) for x, y, z, t; h = u - B l forward, u + B l backward
-  constexpr int W0 = (MU == 0) ? 1 : (MU == 1) ? 0 : (MU == 2) ? 1 : 2;  // power of i in -B, upper row
-  constexpr int W1 = (MU == 0) ? 1 : (MU == 1) ? 2 : (MU == 2) ? 3 : 2;  // lower row
-  constexpr int F = FWD ? 0 : 2;
-  constexpr int r0 = (MU == 0 || MU == 1) ? 1 : 0;                        // spin of l that enters the upper row
-  c2 h[2][3];
-#pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    h[0][a] = addw<(W0 + F) & 3>(f[a], f[6 + 3 * r0 + a]);
-    h[1][a] = addw<(W1 + F) & 3>(f[3 + a], f[6 + 3 * (1 - r0) + a]);
-  }
-  // B^H w = (i w1, i w0), (w1, -w0), (i w0, -i w1), (w0, w1); + forward, - backward
-  constexpr int V0 = (MU == 0) ? 1 : (MU == 1) ? 0 : (MU == 2) ? 1 : 0;
-  constexpr int V1 = (MU == 0) ? 1 : (MU == 1) ? 2 : (MU == 2) ? 3 : 0;
-#pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    c2 w[2];
-#pragma unroll
-    for (int s = 0; s < 2; ++s) {
-      // the products with a minus sign are summed apart and subtracted once
-      float2 pos, neg, sum;
-      if (FWD) {  // sum_c U[a][c] h_c
-        const float2 m0 = m[3 * a], m1 = m[3 * a + 1], m2 = m[3 * a + 2];
-        pos = __ffma2_rn(f2(m2.x), h[s][2].re, __ffma2_rn(f2(m1.x), h[s][1].re, __fmul2_rn(f2(m0.x), h[s][0].re)));
-        neg = __ffma2_rn(f2(m2.y), h[s][2].im, __ffma2_rn(f2(m1.y), h[s][1].im, __fmul2_rn(f2(m0.y), h[s][0].im)));
-        sum = __ffma2_rn(f2(m2.x), h[s][2].im, __ffma2_rn(f2(m1.x), h[s][1].im, __fmul2_rn(f2(m0.x), h[s][0].im)));
-        sum = __ffma2_rn(f2(m2.y), h[s][2].re, __ffma2_rn(f2(m1.y), h[s][1].re, __ffma2_rn(f2(m0.y), h[s][0].re, sum)));
-        w[s] = c2{sub2(pos, neg), sum};
-      } else {  // sum_c conj(U[c][a]) h_c
-        const float2 m0 = m[a], m1 = m[3 + a], m2 = m[6 + a];
-        pos = __ffma2_rn(f2(m2.x), h[s][2].im, __ffma2_rn(f2(m1.x), h[s][1].im, __fmul2_rn(f2(m0.x), h[s][0].im)));
-        neg = __ffma2_rn(f2(m2.y), h[s][2].re, __ffma2_rn(f2(m1.y), h[s][1].re, __fmul2_rn(f2(m0.y), h[s][0].re)));
-        sum = __ffma2_rn(f2(m2.x), h[s][2].re, __ffma2_rn(f2(m1.x), h[s][1].re, __fmul2_rn(f2(m0.x), h[s][0].re)));
-        sum = __ffma2_rn(f2(m2.y), h[s][2].im, __ffma2_rn(f2(m1.y), h[s][1].im, __ffma2_rn(f2(m0.y), h[s][0].im, sum)));
-        w[s] = c2{sum, sub2(pos, neg)};
-      }
+    for (int k = 0; k < 4; ++k) {
+      const float4 v = __ldg(q + k);
+      m[2 * k] = make_float2(v.x, v.y);
+      m[2 * k + 1] = make_float2(v.z, v.w);
     }
-    Su[0][a] = addw<0>(Su[0][a], w[0]);
-    Su[1][a] = addw<0>(Su[1][a], w[1]);
-    Sl[0][a] = addw<(V0 + F) & 3>(Sl[0][a], w[r0]);
-    Sl[1][a] = addw<(V1 + F) & 3>(Sl[1][a], w[1 - r0]);
+    m[8] = __ldg(Ul + 8);
+  }
+  // -B = (i, i), (1, -1), (i, -i), (-1, -1) on the partner row for x, y, z, t, B^H its conjugate transpose's inverse
+  // order: (i, i) on l's rows, (-1, 1), (i, -i), (1, 1) as seen from the row that holds w
+  const float2 one = f2(1.f), mone = f2(-1.f);
+  const float2 s = FWD ? (MU == 0 ? one : MU == 3 ? mone : ln.sg) : (MU == 0 ? mone : MU == 3 ? one : ln.ng);
+  const float2 n = FWD ? (MU == 0 ? mone : MU == 3 ? one : ln.ng) : (MU == 0 ? one : MU == 3 ? mone : ln.sg);
+#pragma unroll
+  for (int a = 0; a < 3; ++a) h[a] = (MU == 0 || MU == 2) ? addi(h[a], l[a], s, n) : adds(h[a], l[a], s);
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    // the products with a minus sign are summed apart and subtracted once
+    float2 pos, neg, sum;
+    c2 w;
+    if (FWD) {  // sum_c U[a][c] h_c
+      const float2 m0 = m[3 * a], m1 = m[3 * a + 1], m2 = m[3 * a + 2];
+      pos = __ffma2_rn(f2(m2.x), h[2].re, __ffma2_rn(f2(m1.x), h[1].re, __fmul2_rn(f2(m0.x), h[0].re)));
+      neg = __ffma2_rn(f2(m2.y), h[2].im, __ffma2_rn(f2(m1.y), h[1].im, __fmul2_rn(f2(m0.y), h[0].im)));
+      sum = __ffma2_rn(f2(m2.x), h[2].im, __ffma2_rn(f2(m1.x), h[1].im, __fmul2_rn(f2(m0.x), h[0].im)));
+      sum = __ffma2_rn(f2(m2.y), h[2].re, __ffma2_rn(f2(m1.y), h[1].re, __ffma2_rn(f2(m0.y), h[0].re, sum)));
+      w = c2{sub2(pos, neg), sum};
+    } else {  // sum_c conj(U[c][a]) h_c
+      const float2 m0 = m[a], m1 = m[3 + a], m2 = m[6 + a];
+      pos = __ffma2_rn(f2(m2.x), h[2].im, __ffma2_rn(f2(m1.x), h[1].im, __fmul2_rn(f2(m0.x), h[0].im)));
+      neg = __ffma2_rn(f2(m2.y), h[2].re, __ffma2_rn(f2(m1.y), h[1].re, __fmul2_rn(f2(m0.y), h[0].re)));
+      sum = __ffma2_rn(f2(m2.x), h[2].re, __ffma2_rn(f2(m1.x), h[1].re, __fmul2_rn(f2(m0.x), h[0].re)));
+      sum = __ffma2_rn(f2(m2.y), h[2].im, __ffma2_rn(f2(m1.y), h[1].im, __ffma2_rn(f2(m0.y), h[0].im, sum)));
+      w = c2{sum, sub2(pos, neg)};
+    }
+    Su[a] = adds(Su[a], w, one);
+    if (MU == 0) L[a] = addi(L[a], w, FWD ? one : mone, FWD ? mone : one);
+    if (MU == 1) L[a] = adds(L[a], w, FWD ? ln.ng : ln.sg);
+    if (MU == 2) L[a] = addi(L[a], w, FWD ? ln.sg : ln.ng, FWD ? ln.ng : ln.sg);
+    if (MU == 3) L[a] = adds(L[a], w, FWD ? one : mone);
   }
 }
 
@@ -187,47 +252,73 @@ __device__ __forceinline__ EoSite eo_site(const Geom &g, int h, int q) {
 }
 __device__ __forceinline__ int eo_lex(const EoSite &s) { return 2 * s.h + (s.x & 1); }
 
-// (H psi)(s) without its signs on the lower spins: upper part Su, lower part -Sl.
-template <class LD>
-__device__ __forceinline__ void hop_eo(const float2 *__restrict__ U, const LD &in, const Geom &g, const EoSite &s,
-                                       c2 (&Su)[2][3], c2 (&Sl)[2][3]) {
+// This row of (H psi)(s): upper spin Su, and Sl, minus the lower spin.  All lanes of a warp take part.
+// AHEAD: hops whose field loads are issued before they are needed (0 or 1).
+template <int AHEAD, class LN, class LD>
+__device__ __forceinline__ void hop_eo(const LN &ln, const float2 *__restrict__ U, const LD &in, const Geom &g,
+                                       const EoSite &s, c2 (&Su)[3], c2 (&Sl)[3]) {
 #pragma unroll
-  for (int r = 0; r < 2; ++r)
-#pragma unroll
-    for (int a = 0; a < 3; ++a) Su[r][a] = Sl[r][a] = zero2();
-  const int P = in.P;
-  const int c[12] = {0, P, 2 * P, 3 * P, 4 * P, 5 * P, 6 * P, 7 * P, 8 * P, 9 * P, 10 * P, 11 * P};
+  for (int a = 0; a < 3; ++a) Su[a] = Sl[a] = zero2();
   const int hx = g.L[0] >> 1, odd = s.x & 1, h = s.h;
-  const int lex = eo_lex(s);
-  const float2 *Us = U + (int64_t)lex * 36;
-  {
-    // x: the pair (2h, 2h + 1) holds one of the two neighbours
-    const int hf = odd ? (s.x == g.L[0] - 1 ? h - (hx - 1) : h + 1) : h;
-    const int hb = odd ? h : (s.x == 0 ? h + (hx - 1) : h - 1);
-    hop_eo_dir<0, true>(Us, in, hf, c, Su, Sl);
-    hop_eo_dir<0, false>(U + (int64_t)(2 * hb + 1 - odd) * 36, in, hb, c, Su, Sl);
+  constexpr int K = kLink32;
+  const float2 *Us = U + (int64_t)eo_lex(s) * (4 * K);
+  int hf[4], hb[4];
+  // x: the pair (2h, 2h + 1) holds one of the two neighbours
+  hf[0] = odd ? (s.x == g.L[0] - 1 ? h - (hx - 1) : h + 1) : h;
+  hb[0] = odd ? h : (s.x == 0 ? h + (hx - 1) : h - 1);
+  const int sy = hx, sz = sy * g.L[1], st = sz * g.L[2];
+  hf[1] = s.y == g.L[1] - 1 ? h - (g.L[1] - 1) * sy : h + sy;
+  hb[1] = s.y == 0 ? h + (g.L[1] - 1) * sy : h - sy;
+  hf[2] = s.z == g.L[2] - 1 ? h - (g.L[2] - 1) * sz : h + sz;
+  hb[2] = s.z == 0 ? h + (g.L[2] - 1) * sz : h - sz;
+  hf[3] = s.t == g.L[3] - 1 ? h - (g.L[3] - 1) * st : h + st;
+  hb[3] = s.t == 0 ? h + (g.L[3] - 1) * st : h - st;
+#define DTR_BLINK(mu, o) (U + (int64_t)(2 * hb[mu] + (o)) * (4 * K) + (mu) * K)
+  typename LD::Raw r0, r1;
+  r0 = in.load(ln, hf[0], ln.clx);
+  if (AHEAD) r1 = in.load(ln, hb[0], ln.clx);
+  hop_eo_dir<0, true>(ln, Us, in, r0, Su, Sl);
+  (AHEAD ? r0 : r1) = in.load(ln, AHEAD ? hf[1] : hb[0], ln.clx);
+  hop_eo_dir<0, false>(ln, DTR_BLINK(0, 1 - odd), in, r1, Su, Sl);
+  (AHEAD ? r1 : r0) = in.load(ln, AHEAD ? hb[1] : hf[1], ln.clx);
+  hop_eo_dir<1, true>(ln, Us + K, in, r0, Su, Sl);
+  (AHEAD ? r0 : r1) = in.load(ln, AHEAD ? hf[2] : hb[1], AHEAD ? ln.clz : ln.clx);
+  hop_eo_dir<1, false>(ln, DTR_BLINK(1, odd), in, r1, Su, Sl);
+  (AHEAD ? r1 : r0) = in.load(ln, AHEAD ? hb[2] : hf[2], ln.clz);
+  // so far Sl belongs to the partner's row
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    Sl[a].re = LN::other_row(Sl[a].re);
+    Sl[a].im = LN::other_row(Sl[a].im);
   }
-  int st = hx;
-  {
-    const int hf = s.y == g.L[1] - 1 ? h - (g.L[1] - 1) * st : h + st;
-    const int hb = s.y == 0 ? h + (g.L[1] - 1) * st : h - st;
-    hop_eo_dir<1, true>(Us + 9, in, hf, c, Su, Sl);
-    hop_eo_dir<1, false>(U + (int64_t)(2 * hb + odd) * 36 + 9, in, hb, c, Su, Sl);
-  }
-  st *= g.L[1];
-  {
-    const int hf = s.z == g.L[2] - 1 ? h - (g.L[2] - 1) * st : h + st;
-    const int hb = s.z == 0 ? h + (g.L[2] - 1) * st : h - st;
-    hop_eo_dir<2, true>(Us + 18, in, hf, c, Su, Sl);
-    hop_eo_dir<2, false>(U + (int64_t)(2 * hb + odd) * 36 + 18, in, hb, c, Su, Sl);
-  }
-  st *= g.L[2];
-  {
-    const int hf = s.t == g.L[3] - 1 ? h - (g.L[3] - 1) * st : h + st;
-    const int hb = s.t == 0 ? h + (g.L[3] - 1) * st : h - st;
-    hop_eo_dir<3, true>(Us + 27, in, hf, c, Su, Sl);
-    hop_eo_dir<3, false>(U + (int64_t)(2 * hb + odd) * 36 + 27, in, hb, c, Su, Sl);
-  }
+  hop_eo_dir<2, true>(ln, Us + 2 * K, in, r0, Su, Sl);
+  (AHEAD ? r0 : r1) = in.load(ln, AHEAD ? hf[3] : hb[2], ln.clz);
+  hop_eo_dir<2, false>(ln, DTR_BLINK(2, odd), in, r1, Su, Sl);
+  (AHEAD ? r1 : r0) = in.load(ln, AHEAD ? hb[3] : hf[3], ln.clz);
+  hop_eo_dir<3, true>(ln, Us + 3 * K, in, r0, Su, Sl);
+  if (!AHEAD) r1 = in.load(ln, hb[3], ln.clz);
+  hop_eo_dir<3, false>(ln, DTR_BLINK(3, odd), in, r1, Su, Sl);
+#undef DTR_BLINK
 }
+
+// Work items [0, n) of one phase over the grid: full sweeps of the whole grid (neighbouring items run at the same
+// time, so the stencil's neighbours meet in L2), and the remainder spread evenly over the blocks (a last sweep of the
+// first blocks alone would leave the other SMs idle: 8^4 x 16 on 19 blocks is 3.4 sweeps).  The remainder goes by
+// GRAIN items, a whole number of sites.  Runs whole warps, so items up to the next multiple of 32 are visited too.
+template <int T, int GRAIN> struct Sweep {
+  int64_t full, lo, hi;
+  __device__ __forceinline__ explicit Sweep(int64_t n) {
+    const int64_t G = gridDim.x, round = G * T;
+    full = n / round * round;
+    const int64_t ch = ((n - full + GRAIN - 1) / GRAIN + G - 1) / G * GRAIN;
+    lo = full + blockIdx.x * ch;
+    hi = min(n, lo + ch);
+  }
+  template <class F> __device__ __forceinline__ void run(const F &body) const {
+    for (int64_t it = (int64_t)blockIdx.x * T + threadIdx.x; it < full; it += (int64_t)gridDim.x * T) body(it);
+    const int64_t it = lo + threadIdx.x;
+    if ((it & ~(int64_t)31) < hi) body(it);
+  }
+};
 
 }  // namespace dtr

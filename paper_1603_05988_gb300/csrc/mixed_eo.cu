@@ -30,6 +30,16 @@ EoBufs eo_carve(char *w, int64_t V, int b) {
   return B;
 }
 
+// body(h, valid) for the work items of all half-lattice sites, in whole warps (the stencil's lanes exchange values)
+template <class F> __device__ __forceinline__ void for_eo_items(const Geom &g, int logp, const F &body) {
+  const int64_t npair = (int64_t)(g.V >> 1) << logp;
+  for (int64_t it = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; (it & ~(int64_t)31) < 2 * npair;
+       it += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t pr = EoLane<4>::pair_of_item(it);
+    body(pr < npair ? (int)(pr >> logp) : 0, pr < npair);
+  }
+}
+
 // rf = hs * scale * r64 in red-black order (zero in inactive and padding columns)
 __global__ void __launch_bounds__(kBlock) k_eo_scale(const double2 *__restrict__ r64, float2 *__restrict__ rf, Geom g,
                                                      int b, int logb, int64_t half, int bi,
@@ -57,41 +67,42 @@ __global__ void __launch_bounds__(kBlock) k_eo_init(const float2 *__restrict__ U
                                                     Geom g, int b, int P, int logp, float wscale,
                                                     const Scal *__restrict__ outer, Scal *inner, double tol2,
                                                     int maxiter, double hs2, Reduce red) {
-  __shared__ double2 tot[64];
-  const int jp = threadIdx.x & (P - 1);
-  const int64_t items = (int64_t)(g.V >> 1) << logp;
-  const CplxLoad odd{rf + half, P, jp}, even{rf, P, jp};
-  const int c[12] = {0, P, 2 * P, 3 * P, 4 * P, 5 * P, 6 * P, 7 * P, 8 * P, 9 * P, 10 * P, 11 * P};
+  __shared__ double2 tot[2 * 64];
+  const EoLane<4> ln(2 * P, threadIdx.x);
+  const CplxLoad odd{rf + half}, even{rf};
   const float2 wp = f2(wscale), wm = f2(-wscale);
   float2 nrm = f2(0.f);
   double2 acc[2] = {make_double2(0.0, 0.0), make_double2(0.0, 0.0)};
-  for (int64_t it = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; it < items;
-       it += (int64_t)gridDim.x * blockDim.x) {
-    const EoSite s = eo_site(g, (int)(it >> logp), 0);
-    c2 Su[2][3], Sl[2][3], own[12];
-    hop_eo(U, odd, g, s, Su, Sl);
-    even.get(s.h, c, own);
-    const int64_t q = (int64_t)s.h * 12 * P + jp;
+  for_eo_items(g, logp, [&](int h, bool valid) {
+    const EoSite s = eo_site(g, h, 0);
+    c2 H[2][3], own[2][3];
+    hop_eo<0>(ln, U, odd, g, s, H[0], H[1]);
+    even.get(ln, h, ln.clz, own[0], own[1]);
+    if (!valid) return;
+    const int64_t q = (int64_t)h * 12 * P + ln.jp;
 #pragma unroll
-    for (int k = 0; k < 12; ++k) {
-      const c2 hk = k < 6 ? Su[k / 3][k % 3] : Sl[(k - 6) / 3][k % 3];
-      const float2 f = k < 6 ? wp : wm;
-      const c2 v{__ffma2_rn(f, hk.re, own[k].re), __ffma2_rn(f, hk.im, own[k].im)};
-      const typename Pair2<S>::T st = Pair2<S>::narrow(v);
-      r[q + k * P] = st;
-      rhat[q + k * P] = st;
-      p[q + k * P] = st;
-      ((float4 *)e)[q + k * P] = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int k = 0; k < 6; ++k) {
+      const c2 hk = H[k / 3][k % 3], o = own[k / 3][k % 3];
+      const float2 f = k < 3 ? wp : wm;
+      const int64_t i = q + (k < 3 ? ln.cu : ln.clz) + (k % 3) * P;
+      const typename Pair2<S>::T st = Pair2<S>::narrow(c2{__ffma2_rn(f, hk.re, o.re), __ffma2_rn(f, hk.im, o.im)});
+      r[i] = st;
+      rhat[i] = st;
+      p[i] = st;
+      ((float4 *)e)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
       const c2 w = Pair2<S>::widen(st);
       nrm = __ffma2_rn(w.re, w.re, __ffma2_rn(w.im, w.im, nrm));
     }
-  }
+  });
   acc[0].x = (double)nrm.x;
   acc[1].x = (double)nrm.y;
-  if (block_reduce<2>(acc, P, red.partial, red.counter, tot)) {
+  // a thread's column pair is threadIdx.x & (P - 1) up to P = 16; with P = 32 the row bit sits in between
+  const int w = P <= 16 ? P : 64;
+  if (block_reduce<2>(acc, w, red.partial, red.counter, tot)) {
     const int j = threadIdx.x;
     if (j < 2 * P) {
-      const double rho = tot[(j & 1) * P + (j >> 1)].x;
+      const int jp = j >> 1, q = (j & 1) * w;
+      const double rho = P <= 16 ? tot[q + jp].x : tot[q + (jp & 15) + 2 * (jp & 16)].x + tot[q + (jp & 15) + 2 * (jp & 16) + 16].x;
       const int act = j < b ? outer->active[j] : 0;
       inner->active[j] = act;
       inner->rho[j] = make_double2(rho, 0.0);
@@ -128,47 +139,49 @@ __global__ void __launch_bounds__(kBlock) k_eo_accum(const float2 *__restrict__ 
     far = __syncthreads_or(far);
     if (q == 0) gs->sel = (allow_update && far) ? 1 : 0;
   }
-  const int jp = threadIdx.x & (P - 1);
-  const int64_t items = (int64_t)(g.V >> 1) << logp;
-  const CplxLoad even{e, P, jp}, res{rf + half, P, jp};
-  const int c[12] = {0, P, 2 * P, 3 * P, 4 * P, 5 * P, 6 * P, 7 * P, 8 * P, 9 * P, 10 * P, 11 * P};
-  const bool a0 = outer->active[2 * jp] != 0, a1 = b > 1 && outer->active[2 * jp + 1] != 0;
-  const double inv0 = a0 ? 1.0 / (outer->scale[2 * jp] * hs) : 0.0;
-  const double inv1 = a1 ? 1.0 / (outer->scale[2 * jp + 1] * hs) : 0.0;
+  const EoLane<4> ln(2 * P, threadIdx.x);
+  const CplxLoad even{e}, res{rf + half};
+  const bool a0 = outer->active[2 * ln.jp] != 0, a1 = b > 1 && outer->active[2 * ln.jp + 1] != 0;
+  const double inv0 = a0 ? 1.0 / (outer->scale[2 * ln.jp] * hs) : 0.0;
+  const double inv1 = a1 ? 1.0 / (outer->scale[2 * ln.jp + 1] * hs) : 0.0;
   const float2 di = f2(dinv), dh = f2(0.5f * dinv), dmh = f2(-0.5f * dinv);
-  for (int64_t it = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; it < items;
-       it += (int64_t)gridDim.x * blockDim.x) {
-    const EoSite s = eo_site(g, (int)(it >> logp), 1);
-    c2 Su[2][3], Sl[2][3], own[12];
-    hop_eo(U, even, g, s, Su, Sl);
-    res.get(s.h, c, own);
-    const int64_t q = (int64_t)s.h * 12 * P + jp;
+  for_eo_items(g, logp, [&](int h, bool valid) {
+    const EoSite s = eo_site(g, h, 1);
+    c2 H[2][3], eo[2][3], ee[2][3];
+    hop_eo<0>(ln, U, even, g, s, H[0], H[1]);
+    res.get(ln, h, ln.clz, eo[0], eo[1]);
+    even.get(ln, h, ln.clz, ee[0], ee[1]);
+    if (!valid) return;
+    const int64_t q = (int64_t)h * 12 * P + ln.jp;
 #pragma unroll
-    for (int k = 0; k < 12; ++k) {
-      const c2 hk = k < 6 ? Su[k / 3][k % 3] : Sl[(k - 6) / 3][k % 3];
-      const float2 f = k < 6 ? dh : dmh;
-      own[k].re = __ffma2_rn(f, hk.re, __fmul2_rn(di, own[k].re));
-      own[k].im = __ffma2_rn(f, hk.im, __fmul2_rn(di, own[k].im));
-      ((float4 *)(e + half))[q + k * P] = make_float4(own[k].re.x, own[k].im.x, own[k].re.y, own[k].im.y);
+    for (int k = 0; k < 6; ++k) {
+      const c2 hk = H[k / 3][k % 3];
+      c2 &o = eo[k / 3][k % 3];
+      const float2 f = k < 3 ? dh : dmh;
+      o = c2{__ffma2_rn(f, hk.re, __fmul2_rn(di, o.re)), __ffma2_rn(f, hk.im, __fmul2_rn(di, o.im))};
+      ((float4 *)(e + half))[q + (k < 3 ? ln.cu : ln.clz) + (k % 3) * P] = to_cols(o);
     }
+    if (!a0 && !a1) return;
     const int lex = eo_lex(s);
-    if (a0 || a1) {
-      double2 *xo = x + (int64_t)lex * 12 * b + 2 * jp, *xe = x + (int64_t)(lex ^ 1) * 12 * b + 2 * jp;
 #pragma unroll
-      for (int k = 0; k < 12; ++k) {
-        const float4 ev = ((const float4 *)e)[q + k * P];
-        double2 v = xo[k * b], u = xe[k * b];
-        xo[k * b] = make_double2(fma((double)own[k].re.x, inv0, v.x), fma((double)own[k].im.x, inv0, v.y));
-        xe[k * b] = make_double2(fma((double)ev.x, inv0, u.x), fma((double)ev.y, inv0, u.y));
-        if (b > 1) {
-          v = xo[k * b + 1];
-          u = xe[k * b + 1];
-          xo[k * b + 1] = make_double2(fma((double)own[k].re.y, inv1, v.x), fma((double)own[k].im.y, inv1, v.y));
-          xe[k * b + 1] = make_double2(fma((double)ev.z, inv1, u.x), fma((double)ev.w, inv1, u.y));
-        }
+    for (int side = 0; side < 2; ++side) {  // the odd site, then the even one of the pair 2h, 2h + 1
+      double2 *xs = x + (int64_t)(side ? lex ^ 1 : lex) * 12 * b + 2 * ln.jp;
+      double2 v[6][2];
+#pragma unroll
+      for (int k = 0; k < 6; ++k) {
+        const double2 *xp = xs + ((k < 3 ? 0 : 6) + 3 * ln.r + k % 3) * b;
+        v[k][0] = xp[0];
+        if (b > 1) v[k][1] = xp[1];
+      }
+#pragma unroll
+      for (int k = 0; k < 6; ++k) {
+        const c2 d = side ? ee[k / 3][k % 3] : eo[k / 3][k % 3];
+        double2 *xp = xs + ((k < 3 ? 0 : 6) + 3 * ln.r + k % 3) * b;
+        xp[0] = make_double2(fma((double)d.re.x, inv0, v[k][0].x), fma((double)d.im.x, inv0, v[k][0].y));
+        if (b > 1) xp[1] = make_double2(fma((double)d.re.y, inv1, v[k][1].x), fma((double)d.im.y, inv1, v[k][1].y));
       }
     }
-  }
+  });
   if (blockIdx.x == 0 && threadIdx.x < b) {
     outer->iters[threadIdx.x] += inner->iters[threadIdx.x];
     outer->flags[threadIdx.x] |= inner->flags[threadIdx.x] & ~kFlagBreakdown;
@@ -192,7 +205,7 @@ static int inner_t(const dtr_gauge_s *gauge, const EoBufs &B, const Geom &g, int
   ea.sc = inner; ea.partial = red.partial; ea.gs = gs;
   ea.max_iters = maxiter + 1;
   ea.grid = grid;
-  k_eo_init<S><<<reduce_grid((int64_t)g.V / 2 * P, device_sms()), kBlock, 0, st>>>(
+  k_eo_init<S><<<reduce_grid((int64_t)g.V * P, device_sms()), kBlock, 0, st>>>(
       gauge->U32, B.rf, half, ea.r, ea.rhat, ea.p, B.e, g, b, P, ea.logp, ea.wscale, outer, inner, inner_tol2, maxiter,
       hs * hs, red);
   count_launches(1);
@@ -220,7 +233,7 @@ int eo_inner(const dtr_gauge_s *gauge, const EoBufs &B, const Geom &g, int b, do
 void eo_accum(const dtr_gauge_s *gauge, const EoBufs &B, const Geom &g, int b, double m0, double2 *x, Scal *outer,
               const Scal *inner, double hs, GridSync *gs, int allow_update, cudaStream_t st) {
   const int bi = eo_width(b), P = bi / 2;
-  k_eo_accum<<<reduce_grid((int64_t)g.V / 2 * P, device_sms()), kBlock, 0, st>>>(
+  k_eo_accum<<<reduce_grid((int64_t)g.V * P, device_sms()), kBlock, 0, st>>>(
       gauge->U32, B.rf, B.e, (int64_t)(g.V / 2) * 12 * bi, x, g, b, P, log2i(P), (float)(1.0 / (4.0 + m0)), outer,
       inner, hs, gs, allow_update);
   count_launches(1);
