@@ -99,10 +99,29 @@ __global__ void __launch_bounds__(kBlock) k_resid(const typename cplx_t<R>::type
   }
 }
 
+// *flag = 1 if any entry of x is nonzero (or NaN).  Callers hand in zeros for want of a guess: finding that out costs
+// one read of x, the stencil on it ten times that (32^3 x 64 x 16: 1 instead of 19 + 8 ms).
+__global__ void __launch_bounds__(kBlock) k_any_nonzero(const ulonglong2 *__restrict__ x, int64_t n, int *flag) {
+  unsigned long long any = 0;
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  for (; e + 7 * stride < n && !any; e += 8 * stride) {
+    ulonglong2 v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = x[e + u * stride];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) any |= (v[u].x | v[u].y) << 1;  // (the sign of a zero does not count)
+  }
+  for (; e < n && !any; e += stride) any |= (x[e].x | x[e].y) << 1;
+  if (any) atomicOr(flag, 1);
+}
+
 // x == 0: r = z (no stencil); tot = (||z||^2, ||z||^2)
 __global__ void __launch_bounds__(kBlock) k_resid_zero(const double2 *__restrict__ z, double2 *__restrict__ r,
-                                                       int64_t n, int b, Scal *sc, Reduce red) {
+                                                       int64_t n, int b, Scal *sc, Reduce red,
+                                                       const int *run_flag = nullptr, int run_if = 0) {
   __shared__ double2 tot[64];
+  if (run_flag && *(volatile const int *)run_flag != run_if) return;  // not selected (uniform over the grid)
   double2 acc[1] = {make_double2(0.0, 0.0)};
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
     const double2 zz = z[e];
@@ -796,6 +815,20 @@ void enqueue_true_resid(const MixedState &S, int restart, const int *run_flag, i
   count_launches(3);
 }
 
+// r64 = z - A x of the initial guess: one kernel if the caller says that x is zero, five otherwise, which find out
+// whether it is
+void enqueue_first_resid(const MixedState &S, int x_is_zero, cudaStream_t st) {
+  const int64_t n = (int64_t)S.g.V * 12 * S.b;
+  int *nz = &S.gs->x_nonzero;
+  if (!x_is_zero) {
+    k_any_nonzero<<<S.gv, kBlock, 0, st>>>((const ulonglong2 *)S.x, n, nz);
+    count_launches(1);
+  }
+  k_resid_zero<<<S.gv, kBlock, 0, st>>>(S.z, S.r64, n, S.b, S.outer, S.red, x_is_zero ? nullptr : nz, 0);
+  count_launches(1);
+  if (!x_is_zero) enqueue_true_resid(S, 1, nz, 1, st);
+}
+
 // Everything a captured graph holds by address or value.  Every link array is in it: a gauge field
 // freed and made again may get some of its old addresses back and others not.
 struct GraphKey {
@@ -863,10 +896,7 @@ int capture_mixed_graph(const MixedState &S, int x_is_zero, double tol2, int max
   open = 1;
   const int64_t n = (int64_t)S.g.V * 12 * S.b;
   k_scal_init<<<1, 64, 0, cs>>>(S.outer, S.b, tol2, maxiter);
-  if (x_is_zero)
-    k_resid_zero<<<S.gv, kBlock, 0, cs>>>(S.z, S.r64, n, S.b, S.outer, S.red);
-  else
-    enqueue_true_resid(S, 1, nullptr, 0, cs);
+  enqueue_first_resid(S, x_is_zero, cs);
   unsigned long long *devcnt = device_launch_counter();
   k_loop_cond<<<1, 32, 0, cs>>>(h, S.outer, S.gs, (unsigned)kMaxRestarts + 1, 1, devcnt, 0);
   CAP_CHECK(cudaGetLastError());
@@ -1003,10 +1033,10 @@ static int solve_mixed_graph(const MixedState &S, int x_is_zero, double tol2, in
   }
   hit->last_use = ++g_graph_tick;
   DTR_CUDA(cudaGraphLaunch(hit->exec, st));
-  // k_scal_init, first residual (one kernel for x = 0, else split + two residual kernels),
+  // k_scal_init, first residual (one kernel for x = 0, else five),
   // k_loop_cond (+ verification: split + two residual kernels, and its k_loop_cond); the
   // loop bodies count themselves on the device
-  count_launches(3 + (x_is_zero ? 0 : 2) + (S.upd ? 4 : 0));
+  count_launches(3 + (x_is_zero ? 0 : 4) + (S.upd ? 4 : 0));
   ++g_graph_launches;
   return DTR_OK;
 }
@@ -1129,10 +1159,9 @@ int solve_internal(const dtr_gauge_s *gauge, double m0, double2 *x, const double
     bool upd_phase = resid_update_enabled(store);
     for (int cycle = 0; cycle <= kMaxRestarts; ++cycle) {
       const int restart = cycle < kMaxRestarts;
-      if (cycle == 0 && x_is_zero) {
-        k_resid_zero<<<gv, kBlock, 0, st>>>(z, S.r64, n, b, outer, red);
-        count_launches(1);
-      } else if (cycle > 0 && upd_phase) {
+      if (cycle == 0) {
+        enqueue_first_resid(S, x_is_zero, st);
+      } else if (upd_phase) {
         enqueue_resid_update(S, st);
         enqueue_true_resid(S, restart, &gs->sel, 0, st);
       } else {
