@@ -198,7 +198,7 @@ static int inner_t(const dtr_gauge_s *gauge, const EoBufs &B, const Geom &g, int
   EoArgs<S> ea;
   ea.U = gauge->U32;
   ea.x = B.e;
-  ea.r = (ST *)B.r; ea.rhat = (ST *)B.rhat; ea.p = (ST *)B.p; ea.v = (ST *)B.v; ea.t = (ST *)B.t; ea.w = (ST *)B.w;
+  ea.r = (ST *)B.r; ea.rhat = (ST *)B.rhat; ea.p = (ST *)B.p; ea.v = (ST *)B.v; ea.t = (ST *)B.t; ea.w = (float4 *)B.w;
   ea.g = g; ea.b = bi; ea.logp = log2i(P);
   ea.diag = (float)(4.0 + m0);
   ea.wscale = (float)(0.5 / (4.0 + m0));

@@ -132,7 +132,8 @@ template <typename S, int T> __global__ void __launch_bounds__(T, 1) k_bicgstab_
   float *shw = (float *)smem;
   float4 *sh = (float4 *)smem;
   const int b = a.b;
-  typedef EoLane<row_bit<S>()> LN;
+  typedef EoLane<row_bit<S>()> LA;   // lanes of the phases that gather Krylov vectors
+  typedef EoLane<row_bit<float>()> LN;  // and of those that gather w
   const LN ln(b, threadIdx.x);
   const int P = ln.P, jp = ln.jp;
   const int64_t nh = a.g.V >> 1;
@@ -150,23 +151,24 @@ template <typename S, int T> __global__ void __launch_bounds__(T, 1) k_bicgstab_
   __syncthreads();
   const float2 dg = f2(a.diag), mh = f2(-0.5f), ph = f2(0.5f);
   const float2 wp = f2(a.wscale), wm = f2(-a.wscale);
-  const PairLoad<S> ldp{a.p}, ldw{a.w};
+  const PairLoad<S> ldp{a.p};
+  const PairLoad<float> ldw{a.w};
   // offset of this thread's component k (upper spin 0..2, lower spin 3..5) from its site
   const int own[6] = {ln.cu, ln.cu + P, ln.cu + 2 * P, ln.clz, ln.clz + P, ln.clz + 2 * P};
   // w at an odd site from the hops of the loader's field
-  auto odd_phase = [&](const auto &ld, auto ahead) {
+  auto odd_phase = [&](const auto &ld, const LA &la, auto ahead) {
     pairs.run([&](int64_t it) {
-      const int64_t pr = LN::pair_of_item(it);
+      const int64_t pr = LA::pair_of_item(it);
       const bool valid = pr < npair;
       const EoSite s = eo_site(a.g, valid ? (int)(pr >> a.logp) : 0, 1);
       c2 Su[3], Sl[3];
-      hop_eo<decltype(ahead)::value>(ln, a.U, ld, a.g, s, Su, Sl);
-      ST *w = a.w + (int64_t)s.h * 12 * P + jp;
+      hop_eo<decltype(ahead)::value>(la, a.U, ld, a.g, s, Su, Sl);
+      float4 *w = a.w + (int64_t)s.h * 12 * P + la.jp;
       if (valid) {
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-          w[own[k]] = PS::narrow(scale2(Su[k], wp));
-          w[own[k + 3]] = PS::narrow(scale2(Sl[k], wm));
+          w[la.cu + k * P] = Pair2<float>::narrow(scale2(Su[k], wp));
+          w[la.clz + k * P] = Pair2<float>::narrow(scale2(Sl[k], wm));
         }
       }
     });
@@ -174,7 +176,7 @@ template <typename S, int T> __global__ void __launch_bounds__(T, 1) k_bicgstab_
 
   for (int iter = 0; iter < a.max_iters; ++iter) {
     if (blockIdx.x == 0 && threadIdx.x == 0) a.gs->iters = iter + 1;
-    odd_phase(ldp, std::integral_constant<int, 0>());  // A
+    odd_phase(ldp, LA(b, threadIdx.x), std::integral_constant<int, 0>());  // A
     if (!grid_arrive_wait(a.gs, ++nbar * G, kSpinBudget)) break;
     {
       float2 d[2] = {f2(0.f), f2(0.f)};
@@ -214,10 +216,11 @@ template <typename S, int T> __global__ void __launch_bounds__(T, 1) k_bicgstab_
       __syncthreads();
     }
     {
-      const PairAxpyLoad<S> ld{a.r, a.v, pair_of(ss.alpha, jp, -1.f)};
+      const LA la(b, threadIdx.x);
+      const PairAxpyLoad<S> ld{a.r, a.v, pair_of(ss.alpha, la.jp, -1.f)};
       // the one phase with two fields to load a hop ahead; FP32 storage has no registers left for it (spills of 1 KB:
       // 262 instead of 187 us at 16^3 x 32 x 32), FP16 gains (1691 -> 1602 us at 32^3 x 64 x 16)
-      odd_phase(ld, std::integral_constant<int, sizeof(ST) == 8 ? 1 : 0>());  // C
+      odd_phase(ld, la, std::integral_constant<int, sizeof(ST) == 8 ? 1 : 0>());  // C
     }
     if (!grid_arrive_wait(a.gs, ++nbar * G, kSpinBudget)) break;
     int n_active = 0;

@@ -11,7 +11,9 @@ namespace dtr {
 template <typename S> struct EoArgs {
   const float2 *U;                                // FP32 links [site][mu][3][3]
   float2 *x;                                      // even sites, interleaved complex
-  typename Pair2<S>::T *r, *rhat, *p, *v, *t, *w;  // w on the odd sites, the others on the even ones
+  typename Pair2<S>::T *r, *rhat, *p, *v, *t;     // even sites
+  float4 *w;                                      // odd sites, FP32: S p = D p - H w / 2 cancels down to the smallest
+                                                  // eigenvalue, so a w rounded to 11 bits would cost its digits
   Geom g;
   int b, logp;                                    // columns; log2(b / 2)
   float diag, wscale;                             // D = 4 + m0, 1 / (2 D)
