@@ -309,6 +309,8 @@ int dtr_dslash(dtr_gauge g, double m0, const double *in, double *out, int nrhs, 
     launch_pack<float>((const double2 *)in, a, g->lat.V, nrhs, b, st);
     launch_dslash_df(g->Udf, a, o, geo, b, m0, st);
     launch_unpack<double>(o, (double2 *)out, g->lat.V, nrhs, b, st);
+  } else if (prec == DTR_F64 && b == 1) {
+    launch_dslash<double>(g->U64, (const double2 *)in, (double2 *)out, geo, 1, m0, dagger, st);  // one column: same layout
   } else if (prec == DTR_F64) {
     double2 *a = (double2 *)w, *o = (double2 *)(w + vb);
     launch_pack<double>((const double2 *)in, a, g->lat.V, nrhs, b, st);

@@ -248,32 +248,57 @@ __global__ void __launch_bounds__(256, MINB) k_dslash_half(const H *__restrict__
 }
 
 // complex c of item `it` in an AoSoA half field (units of one complex = 4 bytes)
-__host__ __device__ __forceinline__ int64_t spc(int64_t it, int c) { return spw(it, c >> 2) * 4 + (c & 3); }
 
-// canonical complex128 (column-major N x nrhs) -> AoSoA half field of width b; padding columns zero
+// canonical complex128 (column-major N x nrhs) <-> AoSoA half field of width b = nrhs: a warp moves 32 items (site,
+// column) through shared memory, so both sides are whole lines, and converts on the integer pipe (one element per thread
+// with its own index divisions and FP64 conversions: 161 and 147 us at 32^3 x 64, one column; 74 us of bytes)
+constexpr int kHalfWarps = 8;
+// offset of the first dof of item it in the canonical block
+__device__ __forceinline__ int64_t item_base(int64_t it, int64_t N, int b) {
+  const int64_t s = b == 1 ? it : it / b;
+  return (it - s * b) * N + s * 12;
+}
 template <typename H>
-__global__ void k_pack_half(const double2 *__restrict__ canon, H *__restrict__ out, int64_t V, int nrhs, int b) {
-  const int64_t n = V * b * 12;
-  const int64_t N = V * 12;
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
-    const int c = (int)(e % 12);
-    const int64_t it = e / 12;
-    const int j = (int)(it % b);
-    const int64_t s = it / b;
-    const double2 v = j < nrhs ? canon[(int64_t)j * N + s * 12 + c] : make_double2(0.0, 0.0);
-    out[spc(it, c)] = HalfOps<H>::from_f2(make_float2((float)v.x, (float)v.y));
+__global__ void __launch_bounds__(32 * kHalfWarps)
+    k_pack_half(const double2 *__restrict__ canon, H *__restrict__ out, int64_t V, int b) {
+  __shared__ __align__(16) H sm[kHalfWarps][32 * 12];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int64_t items = V * b, groups = (items + 31) >> 5;
+  for (int64_t g = (int64_t)blockIdx.x * kHalfWarps + w; g < groups; g += (int64_t)gridDim.x * kHalfWarps) {
+    const int64_t base = item_base(g * 32 + lane, V * 12, b);
+#pragma unroll
+    for (int u = 0; u < 12; ++u) {
+      const int e = u * 32 + lane, it = e / 12;
+      const int64_t src = __shfl_sync(0xffffffffu, base, it) + (e - 12 * it);
+      const double2 v = g * 32 + it < items ? canon[src] : make_double2(0.0, 0.0);
+      sm[w][e] = HalfOps<H>::from_f2(f64_to_f32(v));
+    }
+    __syncwarp();
+    const uint4 *mine = (const uint4 *)&sm[w][lane * 12];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) ((uint4 *)out)[(g * 3 + q) * 32 + lane] = mine[q];
+    __syncwarp();
   }
 }
-
 template <typename H>
-__global__ void k_unpack_half(const H *__restrict__ in, double2 *__restrict__ canon, int64_t V, int nrhs, int b) {
-  const int64_t N = V * 12;
-  const int64_t n = N * nrhs;
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t i = e % N;
-    const int j = (int)(e / N);
-    const float2 f = HalfOps<H>::to_f2(in[spc((i / 12) * b + j, (int)(i % 12))]);
-    canon[e] = make_double2((double)f.x, (double)f.y);
+__global__ void __launch_bounds__(32 * kHalfWarps)
+    k_unpack_half(const H *__restrict__ in, double2 *__restrict__ canon, int64_t V, int b) {
+  __shared__ __align__(16) H sm[kHalfWarps][32 * 12];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int64_t items = V * b, groups = (items + 31) >> 5;
+  for (int64_t g = (int64_t)blockIdx.x * kHalfWarps + w; g < groups; g += (int64_t)gridDim.x * kHalfWarps) {
+    const int64_t base = item_base(g * 32 + lane, V * 12, b);
+    uint4 *mine = (uint4 *)&sm[w][lane * 12];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) mine[q] = ((const uint4 *)in)[(g * 3 + q) * 32 + lane];
+    __syncwarp();
+#pragma unroll
+    for (int u = 0; u < 12; ++u) {
+      const int e = u * 32 + lane, it = e / 12;
+      const int64_t dst = __shfl_sync(0xffffffffu, base, it) + (e - 12 * it);
+      if (g * 32 + it < items) canon[dst] = f32_to_f64(HalfOps<H>::to_f2(sm[w][e]));
+    }
+    __syncwarp();
   }
 }
 
@@ -369,14 +394,14 @@ void launch_dslash_half_canon(const void *Uh, const double2 *in, double2 *out, v
   const size_t fb = (half_field_bytes(V, b) + 255) / 256 * 256;
   if (bf16) {
     __nv_bfloat162 *a = (__nv_bfloat162 *)w, *o = (__nv_bfloat162 *)(w + fb);
-    k_pack_half<__nv_bfloat162><<<g1(V * b * 12), 256, 0, st>>>(in, a, V, nrhs, b);
+    k_pack_half<__nv_bfloat162><<<g1(V * b), 32 * kHalfWarps, 0, st>>>(in, a, V, b);
     launch_half_kernel<__nv_bfloat162>((const __nv_bfloat162 *)Uh, a, o, g, b, (float)(4.0 + m0), g1(V * b), st);
-    k_unpack_half<__nv_bfloat162><<<g1(V * 12 * nrhs), 256, 0, st>>>(o, out, V, nrhs, b);
+    k_unpack_half<__nv_bfloat162><<<g1(V * b), 32 * kHalfWarps, 0, st>>>(o, out, V, b);
   } else {
     __half2 *a = (__half2 *)w, *o = (__half2 *)(w + fb);
-    k_pack_half<__half2><<<g1(V * b * 12), 256, 0, st>>>(in, a, V, nrhs, b);
+    k_pack_half<__half2><<<g1(V * b), 32 * kHalfWarps, 0, st>>>(in, a, V, b);
     launch_half_kernel<__half2>((const __half2 *)Uh, a, o, g, b, (float)(4.0 + m0), g1(V * b), st);
-    k_unpack_half<__half2><<<g1(V * 12 * nrhs), 256, 0, st>>>(o, out, V, nrhs, b);
+    k_unpack_half<__half2><<<g1(V * b), 32 * kHalfWarps, 0, st>>>(o, out, V, b);
   }
   count_launches(3);
 }
