@@ -25,4 +25,22 @@ template <typename S> struct EoArgs {
 };
 template <typename S> int launch_persistent_eo(const EoArgs<S> &ea, cudaStream_t st);
 
+// Plain FP64 BiCGStab with true-residual restarts (persist_eo64.cu).  x and z are whole-lattice fields [site][12][b],
+// the others half-lattice ones [h][12][b], b >= 1.
+struct Eo64Args {
+  const double2 *U;                       // FP64 links [site][mu][3][3]
+  double2 *x;                             // initial guess in (ignored if gs->x_nonzero is 0), solution out
+  const double2 *z;
+  double2 *r, *rhat, *p, *v, *t, *w, *ro;  // w, ro on the odd sites
+  Geom g;
+  int b, logb;
+  double diag;
+  Scal *sc;
+  double2 *partial;
+  GridSync *gs;
+  int max_iters, max_cycles;
+  int grid;
+};
+int launch_persistent_eo64(const Eo64Args &ea, cudaStream_t st);
+
 }  // namespace dtr

@@ -1117,6 +1117,26 @@ int solve_internal(const dtr_gauge_s *gauge, double m0, double2 *x, const double
     K.v = (double2 *)w;    w = align256(w + n * sizeof(double2));
     K.t = (double2 *)w;    w = align256(w + n * sizeof(double2));
     double2 *sv = (double2 *)w; w = align256(w + n * sizeof(double2));
+    if (persistent && eo_usable(m0)) {
+      if (!x_is_zero) {
+        k_any_nonzero<<<gv, kBlock, 0, st>>>((const ulonglong2 *)x, n, &gs->x_nonzero);
+        count_launches(1);
+        DTR_LAUNCH_CHECK("initial guess check");
+      }
+      Eo64Args ea;
+      ea.U = gauge->U64;
+      ea.x = x; ea.z = z;
+      ea.r = K.r; ea.ro = K.r + n / 2; ea.rhat = K.rhat; ea.p = K.rhat + n / 2; ea.v = K.p; ea.t = K.p + n / 2;
+      ea.w = K.v;
+      ea.g = g; ea.b = b; ea.logb = logb; ea.diag = 4.0 + m0;
+      ea.sc = outer; ea.partial = red.partial; ea.gs = gs;
+      ea.max_iters = p->maxiter + 1;
+      ea.max_cycles = kMaxRestarts + 2;
+      ea.grid = p->grid;
+      int rc = launch_persistent_eo64(ea, st);
+      if (rc) return rc;
+      return async ? DTR_OK : read_gs_error(gs, st);
+    }
     if (persistent) {
       DTR_CUDA(cudaMemsetAsync(gs, 0, kGridSyncLaunchBytes, st));
       PArgs<double> pa;
