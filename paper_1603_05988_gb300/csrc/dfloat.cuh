@@ -130,20 +130,5 @@ struct F32AsDf : LexIndex {
     return mkc2(dff(v.x), dff(v.y));
   }
 };
-// the same for a field in red-black order, [parity][site >> 1][12][bi]: the even sites first
-struct EoF32AsDf {
-  const float2 *__restrict__ f;
-  int64_t off_self, off_nbr;  // start of the site's own sublattice and of its neighbours'
-  int bi;
-  __device__ __forceinline__ EoF32AsDf(const float2 *q, int parity, int64_t half, int bi_)
-      : f(q), off_self(parity ? half : 0), off_nbr(parity ? 0 : half), bi(bi_) {}
-  __device__ __forceinline__ int64_t nbr(int s, int, int j) const { return off_nbr + (int64_t)(s >> 1) * 12 * bi + j; }
-  __device__ __forceinline__ int64_t self(int s, int, int j) const { return off_self + (int64_t)(s >> 1) * 12 * bi + j; }
-  __device__ __forceinline__ int stride(int) const { return bi; }
-  __device__ __forceinline__ cdf operator()(int64_t idx) const {
-    const float2 v = f[idx];
-    return mkc2(dff(v.x), dff(v.y));
-  }
-};
 
 }  // namespace dtr

@@ -155,36 +155,6 @@ template <typename S> struct PairAxpyLoad {
     }
   }
 };
-// FP32 field stored as interleaved complex columns, [h][12][b] float2
-__device__ __forceinline__ c2 from_cols(float4 v) { return c2{make_float2(v.x, v.z), make_float2(v.y, v.w)}; }
-__device__ __forceinline__ float4 to_cols(c2 v) { return make_float4(v.re.x, v.im.x, v.re.y, v.im.y); }
-struct CplxLoad {
-  struct Raw {
-    float4 u[3], l[3];
-  };
-  const float2 *f;
-  template <class LN> __device__ __forceinline__ Raw load(const LN &ln, int h, int cl) const {
-    const float4 *q = (const float4 *)f + (int64_t)h * 12 * ln.P + ln.jp;
-    Raw w;
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      w.u[k] = q[ln.cu + k * ln.P];
-      w.l[k] = q[cl + k * ln.P];
-    }
-    return w;
-  }
-  __device__ __forceinline__ void value(const Raw &w, c2 (&u)[3], c2 (&l)[3]) const {
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      u[k] = from_cols(w.u[k]);
-      l[k] = from_cols(w.l[k]);
-    }
-  }
-  template <class LN> __device__ __forceinline__ void get(const LN &ln, int h, int cl, c2 (&u)[3], c2 (&l)[3]) const {
-    value(load(ln, h, cl), u, l);
-  }
-};
-
 // ---------------------------------------------------------------- stencil
 // One hop for one spin row: Su += w, L += +-B^H w, w = U h (FWD) or U^H h, h = u - B l (FWD) or u + B l the row of
 // the neighbour's half spinor (raw: its loaded components).

@@ -283,13 +283,12 @@ template <typename S, int T> __global__ void __launch_bounds__(T, 1) k_bicgstab_
       const s2 mal = pair_of(ss.alpha, je, -1.f), mom = pair_of(ss.omega, je, -1.f);
       const bool act0 = ss.active[2 * je] != 0, act1 = ss.active[2 * je + 1] != 0;
       const bool stop = n_active == 0;
-      float4 *X = (float4 *)a.x;
       elems.run([&](int64_t q) {
         if (q >= nel) return;
         const c2 vv = PS::widen(a.v[q]), pp = PS::widen(a.p[q]);
         const c2 s = axpy2(mal, vv, PS::widen(a.r[q]));
         const c2 tt = PS::widen(a.t[q]);
-        X[q] = to_cols(axpy2(om, s, axpy2(al, pp, from_cols(X[q]))));
+        a.x[q] = Pair2<float>::narrow(axpy2(om, s, axpy2(al, pp, Pair2<float>::widen(a.x[q]))));
         if (!stop) {
           const c2 rn = axpy2(mom, tt, s);
           a.r[q] = PS::narrow(rn);

@@ -7,10 +7,10 @@
 namespace dtr {
 
 // S: storage of the Krylov vectors (float, __half, __nv_bfloat16); arithmetic and the iterate are FP32.
-// Fields are half-lattice [h][12][b], b >= 2 (see eo_core.cuh).
+// Fields are half-lattice [h][12][b / 2] pairs, b >= 2 (see eo_core.cuh).
 template <typename S> struct EoArgs {
   const float2 *U;                                // FP32 links [site][mu][3][3]
-  float2 *x;                                      // even sites, interleaved complex
+  float4 *x;                                      // even sites
   typename Pair2<S>::T *r, *rhat, *p, *v, *t;     // even sites
   float4 *w;                                      // odd sites, FP32: S p = D p - H w / 2 cancels down to the smallest
                                                   // eigenvalue, so a w rounded to 11 bits would cost its digits

@@ -145,8 +145,6 @@ __global__ void __launch_bounds__(kBlock) k_resid_zero(const double2 *__restrict
 // residual (k_resid_df) confirms convergence before the solve reports it.
 // (Two blocks per SM: the register cap spills ~500 B per thread to L1, yet the solve runs ~2% faster
 // than with one block of 255-register threads.)
-// EO: e is in red-black order, [parity][site >> 1][12][max(b, 2)].
-template <bool EO>
 __global__ void __launch_bounds__(kBlock, 2) k_resid_update(const cdf *__restrict__ Udf, const float2 *__restrict__ e,
                                                          double2 *__restrict__ r, Geom g, int b, int logb, dff diag,
                                                          double hs, Scal *sc, Reduce red, const int *run_flag,
@@ -157,17 +155,13 @@ __global__ void __launch_bounds__(kBlock, 2) k_resid_update(const cdf *__restric
   const int64_t n = (int64_t)g.V << logb;
   const int j = threadIdx.x & (b - 1);
   const double inv = sc->active[j] ? 1.0 / (sc->scale[j] * hs) : 0.0;
-  const int bi = b < 2 ? 2 : b;
-  const int64_t half = (int64_t)(g.V >> 1) * 12 * bi;
+  const F32AsDf ld(e);
   for (int64_t it = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; it < n; it += (int64_t)gridDim.x * blockDim.x) {
     const int s = (int)(it >> logb);
     const int64_t base = (int64_t)s * 12 * b + j;
     if (inv != 0.0) {
       cdf o[12], self[12];
-      if (EO)
-        dslash_site_ld<1, dff>(Udf, EoF32AsDf(e, site_parity(g, s), half, bi), g, b, s, j, diag, o, self);
-      else
-        dslash_site_ld<1, dff>(Udf, F32AsDf(e), g, b, s, j, diag, o, self);
+      dslash_site_ld<1, dff>(Udf, ld, g, b, s, j, diag, o, self);
 #pragma unroll
       for (int c = 0; c < 12; ++c) {
         double2 rr = r[base + c * b];
@@ -538,7 +532,7 @@ __global__ void k_scal_init(Scal *sc, int b, double tol2, int maxiter) {
     sc->flags[j] = 0;
     sc->rho[j] = sc->alpha[j] = sc->omega[j] = sc->beta[j] = make_double2(0.0, 0.0);
     sc->rnorm2[j] = sc->bnorm2[j] = sc->rtrue2[j] = 0.0;
-    sc->scale[j] = 1.0;
+    sc->scale[j] = sc->base[j] = sc->fac[j] = 1.0;
   }
   if (j == 0) {
     sc->n_active = 0;
@@ -631,8 +625,8 @@ size_t solver_scratch_bytes(int64_t V, int b, int solver, int gmres_m) {
   const size_t scal = 2 * ((sizeof(Scal) + 255) / 256) * 256;
   const size_t fixed = 256 + red + scal + 256 + 256;
   if (mixed_bicgstab(solver)) {  // half storage uses half of each slot; the larger of the two cycles' buffers
-    const size_t full = 7 * vec32, eo = eo_scratch_bytes(V, b);
-    return fixed + vec64 + (full > eo ? full : eo);
+    const size_t full = vec64 + 7 * vec32, eo = eo_scratch_bytes(V, b);
+    return fixed + (full > eo ? full : eo);
   }
   if (solver == DTR_SOLVER_FGMRES_NET) return fixed + vec64 + 7 * vec32 + fgmres_scratch_bytes(V, b, gmres_m) + 256;
   return fixed + 6 * vec64;
@@ -695,21 +689,18 @@ struct MixedState {
   int store;  // inner Krylov vectors: 0 FP32, 1 FP16, 2 BF16
   double hs;  // inner right-hand-side scale (see k_mixed_init)
   int upd;    // cycles end with the double-float residual update (then one true-residual verification)
-  int eo;     // inner solves on the red-black Schur complement (buffers B), else on the whole lattice (K, sv)
-  EoBufs B;
-  float2 *xhi, *xlo;  // x split for the true residual: idle between inner solves
+  int eo;     // defect correction on the red-black Schur complement (E), else on the whole lattice (r64, K, sv)
+  EoSolve E;
 };
 
 // hands out the buffers of the mixed solvers' cycles from the workspace after the fixed part
 static void carve_mixed(MixedState &S, char *w) {
   const int64_t n = (int64_t)S.g.V * 12 * S.b;
-  S.r64 = (double2 *)w; w = align256(w + n * sizeof(double2));
   if (S.eo) {
-    S.B = eo_carve(w, S.g.V, S.b);
-    S.xhi = (float2 *)S.B.r;          // six half-lattice fields from here on
-    S.xlo = S.xhi + n;
+    S.E = EoSolve{S.gauge, S.g, S.b, S.m0, S.x, S.z, eo_carve(w, S.g.V, S.b), S.outer, S.inner, S.red, S.gs, S.hs, S.grid};
     return;
   }
+  S.r64 = (double2 *)w; w = align256(w + n * sizeof(double2));
   S.K.x = (float2 *)w;    w = align256(w + n * sizeof(float2));
   S.K.r = (float2 *)w;    w = align256(w + n * sizeof(float2));
   S.K.rhat = (float2 *)w; w = align256(w + n * sizeof(float2));
@@ -717,8 +708,6 @@ static void carve_mixed(MixedState &S, char *w) {
   S.K.v = (float2 *)w;    w = align256(w + n * sizeof(float2));
   S.K.t = (float2 *)w;    w = align256(w + n * sizeof(float2));
   S.sv = (float2 *)w;
-  S.xhi = S.K.v;
-  S.xlo = S.K.t;
 }
 
 // inner iterations of one defect-correction cycle on the caller-initialised state
@@ -766,8 +755,7 @@ static int inner_solve(int store, const dtr_gauge_s *gauge, const KrylovVecs<flo
 // Inner solve of one defect-correction cycle after a residual (persistent engine); kernels: those it launched.
 int enqueue_inner(const MixedState &S, cudaStream_t st, int *kernels) {
   if (S.eo) {
-    const int rc = eo_inner(S.gauge, S.B, S.g, S.b, S.m0, S.r64, S.outer, S.inner, S.red, S.gs, S.itol * S.itol,
-                            S.maxiter, S.hs, S.store, S.grid, st, kernels);
+    const int rc = eo_inner(S.E, S.itol * S.itol, S.maxiter, S.store, S.grid, st, kernels);
     *kernels += persist_profile().on ? 1 : 0;
     return rc;
   }
@@ -787,7 +775,7 @@ int enqueue_inner(const MixedState &S, cudaStream_t st, int *kernels) {
 // x += the cycle's correction, choosing the next residual if choose (one kernel)
 void enqueue_accum(const MixedState &S, int choose, cudaStream_t st) {
   if (S.eo) {
-    eo_accum(S.gauge, S.B, S.g, S.b, S.m0, S.x, S.outer, S.inner, S.hs, choose ? S.gs : nullptr, choose, st);
+    eo_accum(S.E, choose, st);
     return;
   }
   k_mixed_accum<<<S.gv, kBlock, 0, st>>>(S.x, S.K.x, (int64_t)S.g.V * 12 * S.b, S.b, S.outer, S.inner, S.hs,
@@ -797,32 +785,40 @@ void enqueue_accum(const MixedState &S, int choose, cudaStream_t st) {
 
 // the double-float residual update, run if gs->sel is 1 (one kernel)
 void enqueue_resid_update(const MixedState &S, cudaStream_t st) {
-  const cdf *U = (const cdf *)S.gauge->Udf;
-  const dff d = split_df(4.0 + S.m0);
-  if (S.eo)
-    k_resid_update<true><<<S.gd, kBlock, 0, st>>>(U, S.B.e, S.r64, S.g, S.b, S.logb, d, S.hs, S.outer, S.red,
-                                                  &S.gs->sel, 1, &S.gs->last_upd);
-  else
-    k_resid_update<false><<<S.gd, kBlock, 0, st>>>(U, S.K.x, S.r64, S.g, S.b, S.logb, d, S.hs, S.outer, S.red,
-                                                   &S.gs->sel, 1, &S.gs->last_upd);
+  if (S.eo) {
+    eo_update(S.E, st);
+    return;
+  }
+  k_resid_update<<<S.gd, kBlock, 0, st>>>((const cdf *)S.gauge->Udf, S.K.x, S.r64, S.g, S.b, S.logb,
+                                          split_df(4.0 + S.m0), S.hs, S.outer, S.red, &S.gs->sel, 1,
+                                          &S.gs->last_upd);
   count_launches(1);
 }
 
 // the true residual (three kernels), run if *run_flag == run_if (NULL: always)
 void enqueue_true_resid(const MixedState &S, int restart, const int *run_flag, int run_if, cudaStream_t st) {
-  launch_true_resid_df(S.gauge, S.x, S.z, S.r64, S.xhi, S.xlo, S.g, S.b, S.logb, S.m0, S.outer, S.red, restart,
+  if (S.eo) {
+    eo_true_resid(S.E, restart, run_flag, run_if, st);
+    return;
+  }
+  launch_true_resid_df(S.gauge, S.x, S.z, S.r64, S.K.v, S.K.t, S.g, S.b, S.logb, S.m0, S.outer, S.red, restart,
                        run_flag, run_if, &S.gs->last_upd, &S.gs->fp64_cert, S.gd, S.gv, st);
   count_launches(3);
 }
 
-// r64 = z - A x of the initial guess: one kernel if the caller says that x is zero, five otherwise, which find out
-// whether it is
+// Residual of the initial guess; where the caller does not say that x is zero the device finds out.
+// first_resid_kernels: the launches.
+int first_resid_kernels(const MixedState &S, int x_is_zero) { return (S.eo ? 2 : 1) + (x_is_zero ? 0 : 4); }
 void enqueue_first_resid(const MixedState &S, int x_is_zero, cudaStream_t st) {
   const int64_t n = (int64_t)S.g.V * 12 * S.b;
   int *nz = &S.gs->x_nonzero;
   if (!x_is_zero) {
     k_any_nonzero<<<S.gv, kBlock, 0, st>>>((const ulonglong2 *)S.x, n, nz);
     count_launches(1);
+  }
+  if (S.eo) {
+    eo_first_resid(S.E, x_is_zero, st);
+    return;
   }
   k_resid_zero<<<S.gv, kBlock, 0, st>>>(S.z, S.r64, n, S.b, S.outer, S.red, x_is_zero ? nullptr : nz, 0);
   count_launches(1);
@@ -1033,10 +1029,10 @@ static int solve_mixed_graph(const MixedState &S, int x_is_zero, double tol2, in
   }
   hit->last_use = ++g_graph_tick;
   DTR_CUDA(cudaGraphLaunch(hit->exec, st));
-  // k_scal_init, first residual (one kernel for x = 0, else five),
+  // k_scal_init, first residual,
   // k_loop_cond (+ verification: split + two residual kernels, and its k_loop_cond); the
   // loop bodies count themselves on the device
-  count_launches(3 + (x_is_zero ? 0 : 4) + (S.upd ? 4 : 0));
+  count_launches(2 + first_resid_kernels(S, x_is_zero) + (S.upd ? 4 : 0));
   ++g_graph_launches;
   return DTR_OK;
 }

@@ -15,6 +15,8 @@ constexpr double kInnerTolFloorBF16 = 1e-2;  // and of BF16-stored ones
 struct Scal {
   double2 rho[64], alpha[64], omega[64], beta[64];
   double rnorm2[64], bnorm2[64], rtrue2[64], scale[64];
+  double base[64], fac[64];  // red-black defect correction: powers of two that scale the residual as it is kept, and
+                             // that to the inner right-hand side (0: column not iterated)
   int active[64], iters[64], restarts[64], conv[64], flags[64];
   int n_active;
   int maxiter;
