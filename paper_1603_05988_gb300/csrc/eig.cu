@@ -140,40 +140,51 @@ __global__ void k_eig_cheb(const C *__restrict__ SY1, const C *__restrict__ Y1, 
 
 // ------------------------------------------------------------------- Gram
 // partial[(chunk * na + ia) * nb + jb] = sum over the chunk's dofs i of
-// conj(A[i, a0 + ia]) B[i, b0 + jb]; 64 x 64 output tiles, 256 threads, each
-// a 4 x 4 sub-tile (rows ty + 16 r, columns tx + 16 c); 16 dofs per shared-memory
+// conj(A[i, a0 + ia]) B[i, b0 + jb]; output tiles of 16 RT by 16 RT, 256 threads, each
+// an RT x RT sub-tile (rows ty + 16 r, columns tx + 16 c); 16 dofs per shared-memory
 // step; FP32 sums over runs of kFlush dofs, added into FP64 (FP64 throughout
 // for FP64 storage).  blockIdx.x = tile (fast), blockIdx.y = dof chunk, so the
-// CTAs in flight share a chunk's rows through L2.
+// CTAs in flight share a chunk's rows through L2.  With sym (A = B) the tiles below
+// the diagonal are left to the reduction, which mirrors them.
+//
+// FP64 storage takes RT = 1: the FP64 pipe (two lanes a clock) bounds it, not shared
+// memory, so what counts is that no padding is computed (basis sizes are multiples of
+// 16; 80 columns in 64-wide tiles are 2.6 times the work) and that enough chunks keep
+// every SM busy: 8^4, 80 columns, 17 ms a product with 64-wide tiles on 48 blocks.
+// FP32 and BF16 storage take RT = 4, bound by shared memory and the FP32 pipe.
 constexpr int kGT = 64, kGK = 16, kFlush = 512;
-template <typename T>
+template <typename T> constexpr int gram_rt() { return sizeof(typename EigAcc<T>::real) == 8 ? 1 : kGT / 16; }
+template <typename T, int RT>
 __global__ void __launch_bounds__(256)
     k_eig_gram(const T *__restrict__ A, int pa, int a0, int na, const T *__restrict__ B, int pb, int b0, int nb,
-               int64_t N, int nchunks, double2 *__restrict__ partial) {
+               int64_t N, int nchunks, int sym, double2 *__restrict__ partial) {
   typedef typename EigAcc<T>::type AC;
   typedef typename EigAcc<T>::real AR;
-  __shared__ AC As[kGK][kGT], Bs[kGK][kGT];
-  const int tilesb = (nb + kGT - 1) / kGT;
+  constexpr int GT = 16 * RT;
+  __shared__ AC As[kGK][GT], Bs[kGK][GT];
+  const int tilesb = (nb + GT - 1) / GT;
   const int ti = blockIdx.x / tilesb, tj = blockIdx.x % tilesb;
+  if (sym && ti > tj) return;
   const int chunk = blockIdx.y;
   const int64_t i0 = N * chunk / nchunks, i1 = N * (chunk + 1) / nchunks;
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  AC acc[4][4];
-  double2 tot[4][4];
+  AC acc[RT][RT];
+  double2 tot[RT][RT];
 #pragma unroll
-  for (int r = 0; r < 4; ++r)
+  for (int r = 0; r < RT; ++r)
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
+    for (int c = 0; c < RT; ++c) {
       acc[r][c].x = acc[r][c].y = 0;
       tot[r][c] = make_double2(0.0, 0.0);
     }
   int since = 0;
   for (int64_t k0 = i0; k0 < i1; k0 += kGK) {
     __syncthreads();
-    for (int q = threadIdx.x; q < kGK * kGT; q += 256) {
-      const int kk = q / kGT, cc = q % kGT;
+#pragma unroll
+    for (int q0 = 0; q0 < kGK * GT; q0 += 256) {
+      const int q = q0 + threadIdx.x, kk = q / GT, cc = q % GT;
       const int64_t i = k0 + kk;
-      const int ca = ti * kGT + cc, cb = tj * kGT + cc;
+      const int ca = ti * GT + cc, cb = tj * GT + cc;
       AC va, vb;
       va.x = va.y = 0;
       vb.x = vb.y = 0;
@@ -187,15 +198,15 @@ __global__ void __launch_bounds__(256)
     __syncthreads();
 #pragma unroll
     for (int kk = 0; kk < kGK; ++kk) {
-      AC a[4], bv[4];
+      AC a[RT], bv[RT];
 #pragma unroll
-      for (int r = 0; r < 4; ++r) a[r] = As[kk][ty + 16 * r];
+      for (int r = 0; r < RT; ++r) a[r] = As[kk][ty + 16 * r];
 #pragma unroll
-      for (int c = 0; c < 4; ++c) bv[c] = Bs[kk][tx + 16 * c];
+      for (int c = 0; c < RT; ++c) bv[c] = Bs[kk][tx + 16 * c];
 #pragma unroll
-      for (int r = 0; r < 4; ++r)
+      for (int r = 0; r < RT; ++r)
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
+        for (int c = 0; c < RT; ++c) {
           // conj(a) b
           acc[r][c].x = fma(a[r].x, bv[c].x, fma(a[r].y, bv[c].y, acc[r][c].x));
           acc[r][c].y = fma(a[r].x, bv[c].y, fma(-a[r].y, bv[c].x, acc[r][c].y));
@@ -204,9 +215,9 @@ __global__ void __launch_bounds__(256)
     since += kGK;
     if (since >= kFlush || k0 + kGK >= i1) {
 #pragma unroll
-      for (int r = 0; r < 4; ++r)
+      for (int r = 0; r < RT; ++r)
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
+        for (int c = 0; c < RT; ++c) {
           tot[r][c].x += (double)acc[r][c].x;
           tot[r][c].y += (double)acc[r][c].y;
           acc[r][c].x = acc[r][c].y = (AR)0;
@@ -215,21 +226,47 @@ __global__ void __launch_bounds__(256)
     }
   }
 #pragma unroll
-  for (int r = 0; r < 4; ++r)
+  for (int r = 0; r < RT; ++r)
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      const int ia = ti * kGT + ty + 16 * r, jb = tj * kGT + tx + 16 * c;
+    for (int c = 0; c < RT; ++c) {
+      const int ia = ti * GT + ty + 16 * r, jb = tj * GT + tx + 16 * c;
       if (ia < na && jb < nb) partial[((int64_t)chunk * na + ia) * nb + jb] = tot[r][c];
     }
 }
 
-// out[e] = sum over chunks (in order) of partial[chunk][e]
-__global__ void k_eig_gram_reduce(const double2 *__restrict__ partial, int64_t ne, int nchunks,
-                                  double2 *__restrict__ out) {
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < ne; e += (int64_t)gridDim.x * blockDim.x) {
+// out[e] = sum over chunks of partial[chunk][e], e < na nb, in one fixed order: 8 threads an element, each a run of
+// chunks; with sym the elements of tiles (GT wide) below the diagonal are the conjugates of those above
+__global__ void __launch_bounds__(256) k_eig_gram_reduce(const double2 *__restrict__ partial, int na, int nb,
+                                                         int nchunks, int sym, int GT, double2 *__restrict__ out) {
+  __shared__ double2 sh[8][32];
+  const int64_t ne = (int64_t)na * nb;
+  const int lane = threadIdx.x & 31, sl = threadIdx.x >> 5;
+  const int lo = nchunks * sl / 8, hi = nchunks * (sl + 1) / 8;
+  for (int64_t e0 = (int64_t)blockIdx.x * 32; e0 < ne; e0 += (int64_t)gridDim.x * 32) {
+    const int64_t e = e0 + lane;
+    const int i = (int)(e / nb), j = (int)(e - (int64_t)i * nb);
+    const bool mirror = sym && i / GT > j / GT;
+    const int64_t src = mirror ? (int64_t)j * nb + i : e;
     double2 s = make_double2(0.0, 0.0);
-    for (int c = 0; c < nchunks; ++c) s = cadd(s, partial[(int64_t)c * ne + e]);
-    out[e] = s;
+    if (e < ne) {
+      int c = lo;
+      for (; c + 3 < hi; c += 4) {
+        double2 v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) v[u] = partial[(int64_t)(c + u) * ne + src];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) s = cadd(s, v[u]);
+      }
+      for (; c < hi; ++c) s = cadd(s, partial[(int64_t)c * ne + src]);
+    }
+    sh[sl][lane] = s;
+    __syncthreads();
+    if (sl == 0 && e < ne) {
+      for (int q = 1; q < 8; ++q) s = cadd(s, sh[q][lane]);
+      if (mirror) s.y = -s.y;
+      out[e] = s;
+    }
+    __syncthreads();
   }
 }
 
@@ -416,9 +453,14 @@ static EigLayout eig_layout(const dtr_lattice_s &lat, const dtr_eig_params *P) {
   const int64_t N = lat.N;
   const size_t es = elem_bytes(P->store);
   const size_t cs = P->store == DTR_F64 ? 16 : 8;  // chunk fields: FP64 or FP32 arithmetic
-  const int tiles = ((L.p + kGT - 1) / kGT) * ((L.p + kGT - 1) / kGT);
+  // dof chunks of a Gram product: enough blocks for four to an SM, each with a run of dofs long enough to outweigh
+  // its partial sums (16-wide FP64 tiles take 16 dofs in as many FP64 instructions as their sums take loads)
+  const int GT = P->store == DTR_F64 ? 16 * gram_rt<double2>() : kGT;
+  const int tiles = ((L.p + GT - 1) / GT) * ((L.p + GT - 1) / GT);
+  const int run = P->store == DTR_F64 ? 256 : 4096;
   int64_t nk = (4LL * device_sms() + tiles - 1) / tiles;
-  const int64_t maxk = N / 4096 > 0 ? N / 4096 : 1;
+  if (P->store == DTR_F64 && nk < 8) nk = 8;
+  const int64_t maxk = N / run > 0 ? N / run : 1;
   if (nk > maxk) nk = maxk;
   if (nk < 1) nk = 1;
   L.nk = (int)nk;
@@ -441,10 +483,13 @@ size_t eig_workspace_bytes(const dtr_lattice_s &lat, const dtr_eig_params *P) { 
 template <typename T>
 static int eig_gram(const T *A, int a0, int na, const T *B, int b0, int nb, int p, int64_t N, int nk,
                     double2 *partial, double2 *out, cudaStream_t st) {
-  const int tiles = ((na + kGT - 1) / kGT) * ((nb + kGT - 1) / kGT);
-  k_eig_gram<T><<<dim3(tiles, nk), 256, 0, st>>>(A, p, a0, na, B, p, b0, nb, N, nk, partial);
+  constexpr int RT = gram_rt<T>(), GT = 16 * RT;
+  const int tiles = ((na + GT - 1) / GT) * ((nb + GT - 1) / GT);
+  const int sym = A == B && a0 == b0 && na == nb;
+  k_eig_gram<T, RT><<<dim3(tiles, nk), 256, 0, st>>>(A, p, a0, na, B, p, b0, nb, N, nk, sym, partial);
   count_launches(1);
-  k_eig_gram_reduce<<<grid_for((int64_t)na * nb), 256, 0, st>>>(partial, (int64_t)na * nb, nk, out);
+  const int64_t blocks = ((int64_t)na * nb + 31) / 32;
+  k_eig_gram_reduce<<<(unsigned)(blocks < 4096 ? blocks : 4096), 256, 0, st>>>(partial, na, nb, nk, sym, GT, out);
   count_launches(1);
   DTR_LAUNCH_CHECK("eigensolver Gram");
   return DTR_OK;
