@@ -12,6 +12,7 @@
 // fixed order, so results are bit-reproducible.
 #include "dtr_internal.cuh"
 #include "deflate.cuh"
+#include "deflate_oz.cuh"
 
 namespace dtr {
 
@@ -21,7 +22,8 @@ constexpr int kMPT = 4;  // vectors m per thread per tile
 template <typename VC>
 __global__ void __launch_bounds__(kDeflBlock)
     k_defl_partial(const VC *__restrict__ Vd, const double2 *__restrict__ Z, int k, int b, int logb, int nsites,
-                   int nchunks, double2 *__restrict__ partial) {
+                   int nchunks, double2 *__restrict__ partial, const int *run_if_set) {
+  if (run_if_set && *run_if_set == 0) return;  // the tensor cores did it
   const int G = kDeflBlock >> logb;  // m-groups per block
   const int tile = G * kMPT;
   const int chunk = blockIdx.x % nchunks;
@@ -49,16 +51,9 @@ __global__ void __launch_bounds__(kDeflBlock)
       for (int q = 0; q < kMPT; ++q) {
         if (!ok[q]) continue;
         const double2 vv = vload(Vd[i * k + m[q]]);
-        const double vx = vv.x, vy = vv.y;
-        // conj(v) * z
-        const double re = vx * z.x + vy * z.y, im = vx * z.y - vy * z.x;
-        if (c < 6) {
-          P[q].x += re;
-          P[q].y += im;
-        } else {
-          Q[q].x += re;
-          Q[q].y += im;
-        }
+        double2 &acc = c < 6 ? P[q] : Q[q];  // += conj(v) z
+        acc.x = fma(vv.x, z.x, fma(vv.y, z.y, acc.x));
+        acc.y = fma(vv.x, z.y, fma(-vv.y, z.x, acc.y));
       }
     }
   }
@@ -250,7 +245,8 @@ __global__ void k_defl_tdg_reduce(const double2 *__restrict__ part, const double
 // x0 (internal [site][12][b]) = V diag(1/lambda) C[:, b:2b]
 template <typename VC>
 __global__ void k_defl_expand(const VC *__restrict__ Vd, const double2 *__restrict__ W, int k, int b, int64_t N,
-                              double2 *__restrict__ x) {
+                              double2 *__restrict__ x, const int *run_if_set) {
+  if (run_if_set && *run_if_set == 0) return;  // the tensor cores did it
   const int64_t n = N * b;
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
     const int j = (int)(e % b);
@@ -336,12 +332,20 @@ size_t defl_scratch_bytes(int64_t V, int k, int b, int sms) {
   if (tc > part) part = tc;
   const size_t C = (size_t)k * 2 * b * sizeof(double2);
   const size_t W = (size_t)k * b * sizeof(double2);
-  const size_t d = 64 * sizeof(double2);
+  const size_t d = 64 * sizeof(double2) + defl_oz_scratch_bytes(k, b) + 256;
   return ((part + 255) / 256 + (C + 255) / 256 + (W + 255) / 256 + (d + 255) / 256 + 5) * 256;
 }
 
 // layout of the scratch: [status word, 256 B][partials][C][x0 weights]
 int *defl_error_word(void *work) { return (int *)(((uintptr_t)work + 255) & ~(uintptr_t)255); }
+
+// Where the digits pay (host-timed calls, FP64 kernels -> digits).  Contraction: 16 sites, FP64 space, k = 96, b = 1
+// 74.7 -> 80.9 us, 256 sites 146 -> 89 us; the FP64 kernel grows by 0.3 us a site in between.
+static bool oz_contract_pays(int64_t V) { return V >= 64; }
+// x0 alone: a tile always has 16 columns, so that one column loses at any size (12x10x6x14, FP32 space, k = 96: b = 1
+// 181 -> 283 us, b = 4 542 -> 311 us), and the setup needs some work to pay (8^4, FP32 space, k = 8: b = 4, 1.6 M products,
+// 37 -> 54 us; b = 16, 6.3 M, 94 -> 74 us).
+static bool oz_expand_pays(int64_t N, int k, int b) { return b >= 4 && N * k * b >= (int64_t)5 << 20; }
 
 int defl_project_internal(const dtr_defl_s *D, const double2 *Z, int b, double2 *d_dev, double2 *terms_dev,
                           double2 *x0_internal, double2 **C_out, void *work, size_t work_bytes, int sms,
@@ -364,6 +368,8 @@ int defl_project_internal(const dtr_defl_s *D, const double2 *Z, int b, double2 
   w += (((size_t)k * 2 * b * sizeof(double2) + 255) / 256) * 256;
   double2 *Wx = (double2 *)w;
   w += (((size_t)k * b * sizeof(double2) + 255) / 256) * 256;
+  void *oz = w;
+  bool contracted = false;  // the digits' scratch is set up by their contraction
   const int logb = log2i(b);
   const int64_t nkb = (int64_t)k * b;
   if (z4 && defl_tc_enabled(D, b)) {
@@ -371,17 +377,26 @@ int defl_project_internal(const dtr_defl_s *D, const double2 *Z, int b, double2 
     int rc = defl_contract_tc(D, Z, b, C, partial, partbytes, err, sms, st, Zc);
     if (rc) return rc;
   } else {
-  if (D->prec == DTR_F64)
-    k_defl_partial<double2><<<nch * tiles, kDeflBlock, 0, st>>>((const double2 *)D->V, Z, k, b, logb, (int)V, nch,
-                                                                partial);
-  else if (D->prec == DTR_F32)
-    k_defl_partial<float2><<<nch * tiles, kDeflBlock, 0, st>>>((const float2 *)D->V, Z, k, b, logb, (int)V, nch,
-                                                               partial);
-  else
-    k_defl_partial<bfc2><<<nch * tiles, kDeflBlock, 0, st>>>((const bfc2 *)D->V, Z, k, b, logb, (int)V, nch,
-                                                             partial);
-  count_launches(1);
-  k_defl_reduce<<<(unsigned)((nkb + 255) / 256), 256, 0, st>>>(partial, k, b, nch, C); count_launches(1);
+    // digits on the tensor cores; where an entry is beyond them (found on the device) the FP64 kernel, on the same chunks
+    int chunks = nch;
+    const int *bad = nullptr;
+    if (D->vexp_ok && oz_contract_pays(V)) {
+      int rc = defl_oz_contract(D, Z, b, oz, nch, partial, &chunks, st);
+      if (rc) return rc;
+      bad = (const int *)oz;
+      contracted = true;
+    }
+    if (D->prec == DTR_F64)
+      k_defl_partial<double2><<<chunks * tiles, kDeflBlock, 0, st>>>((const double2 *)D->V, Z, k, b, logb, (int)V, chunks,
+                                                                     partial, bad);
+    else if (D->prec == DTR_F32)
+      k_defl_partial<float2><<<chunks * tiles, kDeflBlock, 0, st>>>((const float2 *)D->V, Z, k, b, logb, (int)V, chunks,
+                                                                    partial, bad);
+    else
+      k_defl_partial<bfc2><<<chunks * tiles, kDeflBlock, 0, st>>>((const bfc2 *)D->V, Z, k, b, logb, (int)V, chunks,
+                                                                  partial, bad);
+    k_defl_reduce<<<(unsigned)((nkb + 255) / 256), 256, 0, st>>>(partial, k, b, chunks, C);
+    count_launches(2);
   }
   if (d_dev) launch_defl_d(D, C, b, d_dev, terms_dev, st);
   if (x0_internal) {
@@ -389,13 +404,20 @@ int defl_project_internal(const dtr_defl_s *D, const double2 *Z, int b, double2 
     count_launches(1);
     const int64_t n = V * 12 * b;
     unsigned grid = (unsigned)((n + 255) / 256);
-    if (grid > 65535u * 8) grid = 65535u * 8;
+    if (grid > 16u * (unsigned)sms) grid = 16u * (unsigned)sms;
+    const int *bad = nullptr;
+    if (D->vexp_ok && oz_expand_pays(V * 12, k, b)) {
+      if (!contracted) DTR_CUDA(cudaMemsetAsync(oz, 0, 1024, st));
+      int rc = defl_oz_expand(D, Wx, b, oz, x0_internal, st);
+      if (rc) return rc;
+      bad = (const int *)oz;
+    }
     if (D->prec == DTR_F64)
-      k_defl_expand<double2><<<grid, 256, 0, st>>>((const double2 *)D->V, Wx, k, b, V * 12, x0_internal);
+      k_defl_expand<double2><<<grid, 256, 0, st>>>((const double2 *)D->V, Wx, k, b, V * 12, x0_internal, bad);
     else if (D->prec == DTR_F32)
-      k_defl_expand<float2><<<grid, 256, 0, st>>>((const float2 *)D->V, Wx, k, b, V * 12, x0_internal);
+      k_defl_expand<float2><<<grid, 256, 0, st>>>((const float2 *)D->V, Wx, k, b, V * 12, x0_internal, bad);
     else
-      k_defl_expand<bfc2><<<grid, 256, 0, st>>>((const bfc2 *)D->V, Wx, k, b, V * 12, x0_internal);
+      k_defl_expand<bfc2><<<grid, 256, 0, st>>>((const bfc2 *)D->V, Wx, k, b, V * 12, x0_internal, bad);
     count_launches(1);
   }
   DTR_LAUNCH_CHECK("deflation projection");
@@ -430,7 +452,7 @@ int defl_trace_TD(dtr_defl_s *D, cudaStream_t st) {
   if (e != cudaSuccess) return cuda_fail(e, "T_D reduction");
   D->td[0] = h;
   D->td[1] = 0.0;
-  return DTR_OK;
+  return defl_oz_setup(D, st);
 }
 
 int defl_trace_TD_gamma(dtr_defl_s *D, unsigned want, cudaStream_t st) {

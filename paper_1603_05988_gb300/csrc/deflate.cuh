@@ -12,10 +12,8 @@ namespace dtr {
 // exactly to FP64 where the kernels accumulate.
 typedef __nv_bfloat162 bfc2;
 __device__ __forceinline__ double2 vload(const double2 &v) { return v; }
-__device__ __forceinline__ double2 vload(const float2 &v) { return make_double2(v.x, v.y); }
-__device__ __forceinline__ double2 vload(const bfc2 &v) {
-  return make_double2(__bfloat162float(v.x), __bfloat162float(v.y));
-}
+__device__ __forceinline__ double2 vload(const float2 &v) { return f32_to_f64(v); }
+__device__ __forceinline__ double2 vload(const bfc2 &v) { return f32_to_f64(__bfloat1622float2(v)); }
 
 // Scratch for one projection of a width-b block.
 size_t defl_scratch_bytes(int64_t V, int k, int b, int sms);  // includes k x b expansion weights
