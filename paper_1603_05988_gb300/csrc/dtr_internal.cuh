@@ -86,11 +86,14 @@ __host__ __device__ __forceinline__ float2 cmuli(float2 a) { return make_float2(
 // nearest even, exact widening).  The instructions run on the FP64 pipe, at two lanes a clock per SM: converting a field
 // with them takes longer than moving it through HBM (32^3 x 64, one field: 85 us for 50 M values, 74 us for the bytes).
 // What is neither zero nor normal in FP32 goes to the instruction.
+// (the rare cases behind calls: inline, the compiler executes their FP64 instructions every time and selects)
+__device__ __noinline__ static float f64_to_f32_slow(double d) { return __double2float_rn(d); }
+__device__ __noinline__ static double f32_to_f64_slow(float f) { return (double)f; }
 __device__ __forceinline__ float f64_to_f32(double d) {
   const unsigned H = (unsigned)__double2hiint(d), L = (unsigned)__double2loint(d);
   const unsigned sign = H & 0x80000000u, h = H & 0x7fffffffu;
   if ((h | L) == 0u) return __uint_as_float(sign);
-  if (h - 0x38100000u >= 0x0fe00000u) return __double2float_rn(d);  // exponent outside 897 .. 1150
+  if (h - 0x38100000u >= 0x0fe00000u) return f64_to_f32_slow(d);  // exponent outside 897 .. 1150
   const unsigned l = L + (0x0fffffffu + ((L >> 29) & 1u));          // round to nearest even at bit 29
   const unsigned hr = h + (l < L ? 1u : 0u);
   return __uint_as_float(sign | (((hr - 0x38000000u) << 3) | (l >> 29)));
@@ -99,7 +102,7 @@ __device__ __forceinline__ double f32_to_f64(float f) {
   const unsigned b = __float_as_uint(f), m = b & 0x7fffffffu, sign = b & 0x80000000u;
   if (m - 0x00800000u < 0x7f000000u)
     return __hiloint2double((int)(sign | ((m >> 3) + 0x38000000u)), (int)(b << 29));
-  return m == 0u ? __hiloint2double((int)sign, 0) : (double)f;
+  return m == 0u ? __hiloint2double((int)sign, 0) : f32_to_f64_slow(f);
 }
 __device__ __forceinline__ float2 f64_to_f32(double2 v) { return make_float2(f64_to_f32(v.x), f64_to_f32(v.y)); }
 __device__ __forceinline__ double2 f32_to_f64(float2 v) { return make_double2(f32_to_f64(v.x), f32_to_f64(v.y)); }

@@ -97,13 +97,15 @@ __device__ __forceinline__ double pow2_inv(double v) {
   return __hiloint2double((2046 << 20) - (__double2hiint(v) & 0x7ff00000), 0);
 }
 __device__ __forceinline__ int pow2_exp(double v) { return ((__double2hiint(v) >> 20) & 0x7ff) - 1023; }
-// f 2^-e in FP64, exact (integer pipe: a widening by instruction and a fused multiply are two FP64 instructions)
+// f 2^-e in FP64, exact (integer pipe: a widening by instruction and a fused multiply are two FP64 instructions; the
+// rest behind a call, see f64_to_f32)
+__device__ __noinline__ double unscale_slow(float f, int e) { return scalbn((double)f, -e); }
 __device__ __forceinline__ double unscale(float f, int e) {
-  const double d = f32_to_f64(f);
-  const int h = __double2hiint(d), x = ((h >> 20) & 0x7ff) - e;
-  if (f == 0.f) return 0.0;
-  if (x < 1 || x > 2046 || !(fabsf(f) <= 3.4e38f)) return scalbn(d, -e);
-  return __hiloint2double(h - e * (1 << 20), __double2loint(d));
+  const unsigned b = __float_as_uint(f), m = b & 0x7fffffffu;
+  const int x = (int)(m >> 23) + 896 - e;  // exponent field of the result
+  if (m == 0u) return 0.0;
+  if (m - 0x00800000u >= 0x7f000000u || x < 1 || x > 2046) return unscale_slow(f, e);
+  return __hiloint2double((int)((b & 0x80000000u) | ((m >> 3) & 0x000fffffu) | ((unsigned)x << 20)), (int)(b << 29));
 }
 __device__ __forceinline__ void set_fac(Scal *sc, int j, double hs) {
   sc->fac[j] = sc->active[j] ? pow2_below(hs / (sqrt(sc->rtrue2[j]) * sc->base[j])) : 0.0;
@@ -358,7 +360,9 @@ __global__ void __launch_bounds__(kBlock, 2) k_eo_accum(const float2 *__restrict
 // Residual after a cycle without a stencil on x: x grew by e / (base fac), so r -= A e / fac, A e in double-float
 // (links split into hi and lo, e exact in FP32): relative error ~2^-46 of |A| |e|, so r stays the true residual of x
 // to ~1e-14 kappa |z| over all cycles; a true residual confirms convergence before it is reported.
-__global__ void __launch_bounds__(kBlock, 1) k_eo_update(const float4 *__restrict__ Udf, const float4 *__restrict__ e,
+// FP32 arithmetic and load latency bound it: two blocks to an SM (128 registers, ~150 B spilled) 8.9 ms against 9.8 ms for
+// one (232 registers) at 32^3 x 64 x 16; a loop over directions that needs no spills took 10.9 ms.
+__global__ void __launch_bounds__(kBlock, 2) k_eo_update(const float4 *__restrict__ Udf, const float4 *__restrict__ e,
                                                          float4 *__restrict__ rhi, float4 *__restrict__ rlo, Blk k,
                                                          float dhi, float dlo, Scal *sc, Reduce red, double hs,
                                                          const int *run_flag, int run_if, int *mark) {
@@ -398,7 +402,7 @@ __global__ void __launch_bounds__(kBlock, 1) k_eo_update(const float4 *__restric
 
 // True residual r = base (z - A x) with A x in double-float on the split x: each component carries an error of about
 // 2^-46 times the sum of the stencil terms' magnitudes (~9 |x|), i.e. ~1e-13 |x| / |z| relative to z, a hundredth of a
-// 1e-10 tolerance while |x| / |z| stays below ~10.
+// 1e-10 tolerance while |x| / |z| stays below ~10.  One block to an SM: 3.0 ms at 32^3 x 64 x 16, two 3.3 ms.
 __global__ void __launch_bounds__(kBlock, 1) k_eo_resid_df(const float4 *__restrict__ Udf,
                                                            const float4 *__restrict__ xhi,
                                                            const float4 *__restrict__ xlo,
@@ -561,7 +565,7 @@ void eo_accum(const EoSolve &S, int choose, cudaStream_t st) {
 void eo_update(const EoSolve &S, cudaStream_t st) {
   const double D = 4.0 + S.m0;
   const float dh = (float)D;
-  k_eo_update<<<one_per_sm(S), kBlock, 0, st>>>((const float4 *)S.gauge->Udf, S.B.e, S.B.rhi, S.B.rlo, blk_of(S), dh,
+  k_eo_update<<<item_grid(S), kBlock, 0, st>>>((const float4 *)S.gauge->Udf, S.B.e, S.B.rhi, S.B.rlo, blk_of(S), dh,
                                                 (float)(D - (double)dh), S.outer, S.red, S.hs, &S.gs->sel, 1,
                                                 &S.gs->last_upd);
   count_launches(1);
