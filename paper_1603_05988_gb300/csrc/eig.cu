@@ -273,26 +273,29 @@ __global__ void __launch_bounds__(256) k_eig_gram_reduce(const double2 *__restri
 // --------------------------------------------------------------- rotation
 // Y[i, 0:r] <- Y[i, 0:p] Cm (Cm row-major p x r, complex), in place: each CTA
 // takes row blocks of 64 dofs in turn, computes all r outputs tile by tile
-// (64 x 64 tiles, 16-wide steps over p, 4 x 4 per thread) into its own slot
+// (64 x 16 CT tiles, 16-wide steps over p, 4 x CT per thread) into its own slot
 // of `tmp`, then copies the block back.  Columns r .. p-1 are left as they are.
-template <typename T>
+// CT = 4; 1 for FP64 storage, whose pipe is the bound (see the Gram kernel): 80 columns
+// in 64-wide tiles took 3.9 ms at 8^4.
+template <typename T, int CT>
 __global__ void __launch_bounds__(256)
     k_eig_rotate(T *__restrict__ Y, int64_t N, int p, int r, const typename EigAcc<T>::type *__restrict__ Cm,
                  T *__restrict__ tmp) {
   typedef typename EigAcc<T>::type AC;
-  __shared__ AC As[kGK][kGT], Bs[kGK][kGT];
+  constexpr int WT = 16 * CT;
+  __shared__ AC As[kGK][kGT], Bs[kGK][WT];
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
   T *slot = tmp + (int64_t)blockIdx.x * kGT * r;
   const int64_t nblk = (N + kGT - 1) / kGT;
-  const int ctiles = (r + kGT - 1) / kGT;
+  const int ctiles = (r + WT - 1) / WT;
   for (int64_t blk = blockIdx.x; blk < nblk; blk += gridDim.x) {
     const int64_t row0 = blk * kGT;
     for (int ct = 0; ct < ctiles; ++ct) {
-      AC acc[4][4];
+      AC acc[4][CT];
 #pragma unroll
       for (int a = 0; a < 4; ++a)
 #pragma unroll
-        for (int c = 0; c < 4; ++c) acc[a][c].x = acc[a][c].y = 0;
+        for (int c = 0; c < CT; ++c) acc[a][c].x = acc[a][c].y = 0;
       for (int j0 = 0; j0 < p; j0 += kGK) {
         __syncthreads();
         for (int q = threadIdx.x; q < kGK * kGT; q += 256) {
@@ -302,24 +305,26 @@ __global__ void __launch_bounds__(256)
           v.x = v.y = 0;
           if (i < N && j0 + kk < p) v = ldacc(Y[i * p + j0 + kk], (AC *)nullptr);
           As[kk][rr] = v;
-          const int kk2 = q / kGT, cc = q % kGT;
+        }
+        for (int q = threadIdx.x; q < kGK * WT; q += 256) {
+          const int kk2 = q / WT, cc = q % WT;
           AC w;
           w.x = w.y = 0;
-          if (j0 + kk2 < p && ct * kGT + cc < r) w = Cm[(int64_t)(j0 + kk2) * r + ct * kGT + cc];
+          if (j0 + kk2 < p && ct * WT + cc < r) w = Cm[(int64_t)(j0 + kk2) * r + ct * WT + cc];
           Bs[kk2][cc] = w;
         }
         __syncthreads();
 #pragma unroll
         for (int kk = 0; kk < kGK; ++kk) {
-          AC a[4], bv[4];
+          AC a[4], bv[CT];
 #pragma unroll
           for (int q = 0; q < 4; ++q) a[q] = As[kk][ty + 16 * q];
 #pragma unroll
-          for (int c = 0; c < 4; ++c) bv[c] = Bs[kk][tx + 16 * c];
+          for (int c = 0; c < CT; ++c) bv[c] = Bs[kk][tx + 16 * c];
 #pragma unroll
           for (int q = 0; q < 4; ++q)
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
+            for (int c = 0; c < CT; ++c) {
               acc[q][c].x = fma(a[q].x, bv[c].x, fma(-a[q].y, bv[c].y, acc[q][c].x));
               acc[q][c].y = fma(a[q].x, bv[c].y, fma(a[q].y, bv[c].x, acc[q][c].y));
             }
@@ -328,8 +333,8 @@ __global__ void __launch_bounds__(256)
 #pragma unroll
       for (int q = 0; q < 4; ++q)
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          const int rr = ty + 16 * q, m = ct * kGT + tx + 16 * c;
+        for (int c = 0; c < CT; ++c) {
+          const int rr = ty + 16 * q, m = ct * WT + tx + 16 * c;
           if (m < r) slot[(int64_t)rr * r + m] = st2<T>((double)acc[q][c].x, (double)acc[q][c].y);
         }
     }
@@ -717,7 +722,7 @@ static int eig_solve_t(const dtr_gauge_s *gauge, double m0, const dtr_eig_params
     tp = now();
     // Y <- Y C (QY is rebuilt after the next filter, so it is not rotated)
     DTR_CUDA(cudaMemcpyAsync(Cd, hC.data(), sizeof(AC) * (size_t)p * r, cudaMemcpyHostToDevice, st));
-    k_eig_rotate<T><<<L.rot_grid, 256, 0, st>>>(Y, N, p, r, Cd, rtmp);
+    k_eig_rotate<T, gram_rt<T>()><<<L.rot_grid, 256, 0, st>>>(Y, N, p, r, Cd, rtmp);
     count_launches(1);
     int nch = 4 * device_sms();
     if (nch > N) nch = (int)N;
