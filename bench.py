@@ -325,14 +325,18 @@ def run_reference(args):
 
 
 # --------------------------------------------------------------- GPU path
+TRAFFIC_F16_B16 = 748.0
+
+
 def persistent_roofline(prof, sms, lanes, wall_ms, block, hbm_peak, hbm_note, workload, vec_bytes=96):
-    """Roofline of the persistent BiCGStab kernel from its device-timed launches.
-    Algorithmic bytes per site, RHS and iteration: the fused minimum of one BiCGStab
-    iteration, two stencils (a vector in + a vector out + 288 / b B of FP32 links each)
-    and six vector passes, a vector being 96 B per site and RHS in FP32 storage and 48 B
-    in FP16; flops 2 x 1368 + 12 x 104."""
-    bytes_unit = 2 * (2 * vec_bytes + 288.0 / block) + 6 * vec_bytes
-    flop_unit = 2 * 1368.0 + 12 * 104.0
+    """Roofline of the persistent BiCGStab kernel (red-black Schur complement) from its
+    device-timed launches.  Algorithmic bytes per whole-lattice site, RHS and iteration: the
+    fused minimum of one iteration, two applications of the Schur complement (a half-length
+    vector in and one out, 288 / b B of FP32 links each) and six half-length vector passes, a
+    whole vector being 96 B per site and RHS in FP32 storage and 48 B in FP16; flops
+    2 x (1320 + 24) for the hops and the diagonal, 6 x 104 for the vectors."""
+    bytes_unit = 2 * (vec_bytes + 288.0 / block) + 3 * vec_bytes
+    flop_unit = 2 * 1344.0 + 6 * 104.0
     n = max(prof["launches"], 1)
     pms = prof["ms"] / n
     units = prof["site_rhs_iterations"] / n
@@ -342,24 +346,23 @@ def persistent_roofline(prof, sms, lanes, wall_ms, block, hbm_peak, hbm_note, wo
     share = grid / sms
     fp32_peak = sms * 128 * 2 * 2.07e9 / 1e12
     # DRAM bytes per site, RHS and iteration of the same kernel under ncu (16^3x32, 16 RHS, FP16
-    # storage: profiles/persistent_bicgstab_f16_16x16x16x32_b16.md), scaled to this launch's units;
-    # the FP32-storage counters predate the current kernel, so none is given for it
-    traffic, traffic_note = None, "no capture of the current FP32-storage kernel"
+    # storage: profiles/bicgstab_eo_f16_16x16x16x32_b16.md), scaled to this launch's units
+    traffic, traffic_note = None, "captured for FP16 storage and 16 RHS only"
     if vec_bytes == 48 and block == 16:
-        traffic = 848.0 * units
-        traffic_note = ("848 B per site, RHS and iteration (ncu DRAM read + write at 16^3x32, 16 RHS, FP16 storage) "
-                        "x this launch's site-RHS-iterations")
+        traffic = TRAFFIC_F16_B16 * units
+        traffic_note = ("%.0f B per site, RHS and iteration (ncu DRAM read + write at 16^3x32, 16 RHS, FP16 storage) "
+                        "x this launch's site-RHS-iterations" % TRAFFIC_F16_B16)
     return {"bound": "hbm", "achieved": gbs, "peak": hbm_peak * share, "unit": "GB/s", "frac": gbs / (hbm_peak * share),
             "traffic": traffic, "traffic_note": traffic_note,
-            "kernel": "k_bicgstab_persistent (%s-stored inner BiCGStab, %d RHS, %s)"
+            "kernel": "k_bicgstab_eo (%s-stored inner BiCGStab on the Schur complement, %d RHS, %s)"
                                        % ("FP32" if vec_bytes == 96 else "FP16", block, workload),
             "avg_launch_ms": pms, "launches": prof["launches"], "alg_bytes_per_launch": units * bytes_unit,
-            "alg_bytes_note": "%.0f B per site, RHS and iteration (two stencils 2 x (%d + %d + 288/%d) + six "
-                              "%d B vector passes: the fused minimum) x site-RHS-iterations of the launch"
-                              % (bytes_unit, vec_bytes, vec_bytes, block, vec_bytes),
+            "alg_bytes_note": "%.0f B per site, RHS and iteration (two Schur applications 2 x (%d + 288/%d) + six "
+                              "%d B half-length vector passes: the fused minimum) x site-RHS-iterations of the launch"
+                              % (bytes_unit, vec_bytes, block, vec_bytes // 2),
             "peak_note": hbm_note + "; times the launch's SM share %d/%d" % (grid, sms),
             "fp32": {"achieved_tflops": tfl, "peak_tflops": fp32_peak * share, "frac": tfl / (fp32_peak * share),
-                     "note": "3984 flop per site, RHS and iteration; FP32 peak = SMs x 128 x 2 x 2.07 GHz (nominal)"},
+                     "note": "3312 flop per site, RHS and iteration; FP32 peak = SMs x 128 x 2 x 2.07 GHz (nominal)"},
             "aggregate_gbs": prof["site_rhs_iterations"] * bytes_unit / (wall_ms / 1e3) / 1e9 if wall_ms else None,
             "ctas_per_launch": grid, "concurrent_launches": lanes}
 
@@ -711,7 +714,7 @@ def measure_small(args, dtr, synth, torch, barrier, max_over_ranks, sms, hbm_pea
     t_run64 = (sum(ms64) / (nf * L64)) / 1e3
     # roofline: at 8^4 the persistent kernel is L2-resident and latency-bound; against its SM share of FP32
     fp32_peak = sms * 128 * 2 * 2.07e9 / 1e12
-    flop_unit = 2 * 1368.0 + 12 * 104.0
+    flop_unit = 2 * 1344.0 + 6 * 104.0
     n = max(prof["launches"], 1)
     pms = prof["ms"] / n
     achieved = prof["site_rhs_iterations"] * flop_unit / n / (pms / 1e3) / 1e12 if pms > 0 else 0.0
@@ -729,7 +732,7 @@ def measure_small(args, dtr, synth, torch, barrier, max_over_ranks, sms, hbm_pea
                                 "speedup_vs_fp64_path": t_run64 / t_run},
             "roofline": {"bound": "alu", "achieved": achieved, "peak": fp32_peak * grid / sms, "unit": "TFLOP/s",
                          "frac": achieved / (fp32_peak * grid / sms),
-                         "kernel": "k_bicgstab_persistent (FP32 inner solve, 16 RHS, 8^4, L2-resident)",
+                         "kernel": "k_bicgstab_eo (FP32 inner solve on the Schur complement, 16 RHS, 8^4, L2-resident)",
                          "avg_launch_ms": pms, "launches": prof["launches"], "ctas_per_launch": grid},
             "l2": "flushed (256 MiB write) before every timed step"}
 
