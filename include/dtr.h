@@ -264,7 +264,8 @@ int dtr_solve_batch(dtr_gauge g, double m0, const double *z, double *y, int nrhs
  * (non-zero).  The library copies V to device memory in precision prec
  * (DTR_F64, DTR_F32, or DTR_BF16 rounded to nearest even: 4 bytes per
  * complex value) and computes T_D in FP64 from the stored copy; every
- * kernel widens the stored values exactly to FP64, so the estimator stays
+ * kernel works on the stored values, widened exactly to FP64 or, in the tensor-core
+ * projections, as integers (see dtr_deflate_project), so the estimator stays
  * unbiased for the rounded V. */
 int dtr_defl_create(dtr_lattice lat, int k, dtr_prec prec, const double *V_host,
                     const double *lambda_host, dtr_defl *out);
@@ -360,6 +361,10 @@ int dtr_defl_to_host(dtr_defl d, double *V_host, double *lambda_host);
  * coeff_out: device k x 2 nrhs complex128 column-major, or NULL.
  * x0_out: device canonical N x nrhs, or NULL: receives the deflated solution
  *   V diag(1/lambda) V^H gamma_5 z = A_D^-1 z.
+ * Accuracy: that of FP64 sums, C to about 2^-53 of sum |v| |z|.  Larger blocks run on the tensor cores in integers
+ * relative to each column's largest entry, with 54 bits; blocks for which that would lose digits (entries small in V
+ * where z is large or the other way round, point sources, solutions x0 that are small over a whole neighbourhood of 16
+ * dofs; not finite values) are found on the device and take FP64 sums, at the FP64 pipe's rate.
  * work: device workspace of dtr_deflate_workspace_bytes(d, nrhs) bytes. */
 size_t dtr_deflate_workspace_bytes(dtr_defl d, int nrhs);
 int dtr_deflate_project(dtr_defl d, const double *z, int nrhs, double *d_out, double *coeff_out,

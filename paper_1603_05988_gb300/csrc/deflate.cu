@@ -23,7 +23,7 @@ template <typename VC>
 __global__ void __launch_bounds__(kDeflBlock)
     k_defl_partial(const VC *__restrict__ Vd, const double2 *__restrict__ Z, int k, int b, int logb, int nsites,
                    int nchunks, double2 *__restrict__ partial, const int *run_if_set) {
-  if (run_if_set && *run_if_set == 0) return;  // the tensor cores did it
+  if (run_if_set && !(run_if_set[0] | run_if_set[1])) return;  // the tensor cores did it
   const int G = kDeflBlock >> logb;  // m-groups per block
   const int tile = G * kMPT;
   const int chunk = blockIdx.x % nchunks;
@@ -246,7 +246,7 @@ __global__ void k_defl_tdg_reduce(const double2 *__restrict__ part, const double
 template <typename VC>
 __global__ void k_defl_expand(const VC *__restrict__ Vd, const double2 *__restrict__ W, int k, int b, int64_t N,
                               double2 *__restrict__ x, const int *run_if_set) {
-  if (run_if_set && *run_if_set == 0) return;  // the tensor cores did it
+  if (run_if_set && !(run_if_set[0] | run_if_set[1])) return;  // the tensor cores did it
   const int64_t n = N * b;
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
     const int j = (int)(e % b);
@@ -369,7 +369,6 @@ int defl_project_internal(const dtr_defl_s *D, const double2 *Z, int b, double2 
   double2 *Wx = (double2 *)w;
   w += (((size_t)k * b * sizeof(double2) + 255) / 256) * 256;
   void *oz = w;
-  bool contracted = false;  // the digits' scratch is set up by their contraction
   const int logb = log2i(b);
   const int64_t nkb = (int64_t)k * b;
   if (z4 && defl_tc_enabled(D, b)) {
@@ -377,14 +376,13 @@ int defl_project_internal(const dtr_defl_s *D, const double2 *Z, int b, double2 
     int rc = defl_contract_tc(D, Z, b, C, partial, partbytes, err, sms, st, Zc);
     if (rc) return rc;
   } else {
-    // digits on the tensor cores; where an entry is beyond them (found on the device) the FP64 kernel, on the same chunks
+    // digits on the tensor cores; what is beyond them (found on the device) the FP64 kernel does, on the same chunks
     int chunks = nch;
     const int *bad = nullptr;
     if (D->vexp_ok && oz_contract_pays(V)) {
       int rc = defl_oz_contract(D, Z, b, oz, nch, partial, &chunks, st);
       if (rc) return rc;
-      bad = (const int *)oz;
-      contracted = true;
+      bad = defl_oz_contract_flags(oz);
     }
     if (D->prec == DTR_F64)
       k_defl_partial<double2><<<chunks * tiles, kDeflBlock, 0, st>>>((const double2 *)D->V, Z, k, b, logb, (int)V, chunks,
@@ -407,10 +405,9 @@ int defl_project_internal(const dtr_defl_s *D, const double2 *Z, int b, double2 
     if (grid > 16u * (unsigned)sms) grid = 16u * (unsigned)sms;
     const int *bad = nullptr;
     if (D->vexp_ok && oz_expand_pays(V * 12, k, b)) {
-      if (!contracted) DTR_CUDA(cudaMemsetAsync(oz, 0, 1024, st));
       int rc = defl_oz_expand(D, Wx, b, oz, x0_internal, st);
       if (rc) return rc;
-      bad = (const int *)oz;
+      bad = defl_oz_expand_flags(oz);
     }
     if (D->prec == DTR_F64)
       k_defl_expand<double2><<<grid, 256, 0, st>>>((const double2 *)D->V, Wx, k, b, V * 12, x0_internal, bad);

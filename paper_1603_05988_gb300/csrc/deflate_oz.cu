@@ -1,8 +1,8 @@
-// Deflation projection of general FP64 blocks on the tensor cores: C = V^H [Z, g5 Z] and x0 = V W with FP64 accuracy
-// from exact integer products.
+// Deflation projection of general FP64 blocks on the tensor cores: C = V^H [Z, g5 Z] and x0 = V W from exact integer
+// products, where that is as accurate as FP64 sums.
 //
 // FP64 runs at two lanes a clock per SM, so the plain contraction costs 8 N k b FP64 instructions (16^3 x 32, k = 64,
-// b = 16: 24 ms, and 17 ms for x0).  Here every real column of V and Z is written as integers of 56 bits times a power
+// b = 16: 24 ms, and 17 ms for x0).  Here every real column of V and Z is written as integers of 54 bits times a power
 // of two (relative to the column's largest entry), the integers as seven balanced base-256 digits (Ozaki, Ogita, Oishi
 // and Rump's error-free splitting, Numer. Algorithms 59, 2012), and the digit products run as BF16 mma with FP32
 // accumulation: a digit is exact in BF16, a product at most 2^14, and 128 of them times the seven digit pairs of one
@@ -10,12 +10,25 @@
 // dropped is 2^-57 of the product of the column maxima, below the rounding of an FP64 sum.  The sums of one weight go to
 // 64-bit integers, and to FP64 once at the end.
 //
+// Integers are fixed point where FP64 floats: an entry is off by up to 2^-55 of its column's largest, so a product of two
+// entries that are both small for their columns loses digits.  Two tests on the device send such blocks to the FP64
+// kernels (a point source; vectors that decay from opposite ends):
+//   C   S = sum of the products of the entries' moduli, in units of the columns' powers of two, must reach
+//       sqrt(n / 2) for n nonzero entries of z (k_oz_mass).  The digits' error is then below 0.06 2^-53 of
+//       sum |v| |z|; FP64 chains come to 0.02 to 0.2 (49152 dofs, 18 families of graded, localised, sparse and plain
+//       columns).  Gaussian columns reach 4.4 sqrt(n) there, growing with sqrt(n).
+//   x0  sixteen neighbouring entries of a column must have an RMS of 2^-7.5 sqrt(k) in the weights' units, 2^-6.5 if V is
+//       FP64 (k_oz_expand).  Their error is then below 2^-50 of their norm (largest seen 6e-16; FP64 sums 1e-15 at
+//       k = 200).  Gaussian V and weights over three decades reach 2^-6.2 and more.
+//
 // Digits come from shifts and byte permutes on the integer pipe.  A digit plane of Z that is zero over a stage is
 // skipped: probing noise (entries 0, +-1, +-i) has one digit.
 //
 // 16^3 x 32, FP32 space, k = 64, b = 16, with x0: 42.0 -> 5.7 ms.  Relative error against exact sums there: x0
 // 4.8e-16 -> 1.6e-16, C 8.6e-17 -> 8.5e-17 (the FP64 kernels add in a chain).
 #include "deflate_oz.cuh"
+
+#include <cmath>
 
 namespace dtr {
 
@@ -94,19 +107,23 @@ __device__ __forceinline__ bool is_zero(double2 v) {
 }
 __device__ __forceinline__ bool is_zero(bfc2 v) { return is_zero(__bfloat1622float2(v)); }
 
-// stat[c]: 0 while the column is all zeros, else 1 + the largest exponent field
+// stat[c]: 0 while the column is all zeros, else 1 + the largest exponent field; count[c] (or NULL): nonzero entries
 template <typename T>
-__global__ void __launch_bounds__(256) k_oz_exp(const T *__restrict__ F, int64_t rows, int cols, int *__restrict__ stat) {
+__global__ void __launch_bounds__(256)
+    k_oz_exp(const T *__restrict__ F, int64_t rows, int cols, int *__restrict__ stat, int *__restrict__ count) {
   for (int c0 = 0; c0 < cols; c0 += 256) {
     const int w = min(256, cols - c0), g = 256 / w;  // g rows of w columns at once
     const int c = threadIdx.x % w, r = threadIdx.x / w;
     if (r < g) {
-      int m = 0;
+      int m = 0, n = 0;
       for (int64_t i = (int64_t)blockIdx.x * g + r; i < rows; i += (int64_t)gridDim.x * g) {
         const T v = F[i * cols + c0 + c];
-        if (!is_zero(v)) m = max(m, 1 + exp_field(v));
+        if (is_zero(v)) continue;
+        m = max(m, 1 + exp_field(v));
+        ++n;
       }
-      if (m) atomicMax(&stat[c0 + c], m);  // (the largest does not depend on the order)
+      if (m) atomicMax(&stat[c0 + c], m);  // (neither the largest nor the count depends on the order)
+      if (n && count) atomicAdd(&count[c0 + c], n);
     }
   }
 }
@@ -203,6 +220,94 @@ __device__ __forceinline__ void step(Acc &s, unsigned a, unsigned pa, unsigned b
   }
 }
 
+// ------------------------------------------------------------------- mass
+// largest of |re|, |im| times 2^-e as BF16 bits, rounded down (0 below 2^-126)
+__device__ __forceinline__ unsigned mag(float2 v, int e) {
+  const unsigned m = max(__float_as_uint(v.x) & 0x7fffffffu, __float_as_uint(v.y) & 0x7fffffffu);
+  const int x = (int)(m >> 23), r = x - e;
+  return x == 0 || r < 1 ? 0u : (unsigned)r << 7 | (m >> 16 & 0x7fu);
+}
+__device__ __forceinline__ unsigned mag(double2 v, int e) {
+  const unsigned m = max((unsigned)__double2hiint(v.x) & 0x7fffffffu, (unsigned)__double2hiint(v.y) & 0x7fffffffu);
+  const int x = (int)(m >> 20), r = x - 896 - e;
+  return x == 0 || r < 1 ? 0u : (unsigned)r << 7 | (m >> 13 & 0x7fu);
+}
+__device__ __forceinline__ unsigned mag(bfc2 v, int e) { return mag(__bfloat1622float2(v), e); }
+
+// mass[m b + j] += 2^16 sum over sites of |v| |z| (moduli as above: a lower bound, so part of the sites may do); the last
+// block compares with sqrt(n / 2) and sets *fail for a pair that falls short.  Sites: every step-th (REST = false), or all
+// but these (run if *need is set).  A block: 64 vectors x 16 columns, stages of 4 sites as BF16 in shared memory; eight
+// warps of 16 x 8 sums.
+constexpr int kMM = 64, kMJ = 16, kMK = 48;
+constexpr int kMAs = (kMM + 8) * 2, kMBs = (kMJ + 8) * 2;  // bytes of a dof row
+template <typename VC, bool REST>
+__global__ void __launch_bounds__(256)
+    k_oz_mass(const VC *__restrict__ Vd, const int *__restrict__ ev, const double2 *__restrict__ Z,
+              const int *__restrict__ ez, const int *__restrict__ count, const int *__restrict__ bad,
+              const int *__restrict__ need, int k, int b, int nsites, int step, unsigned long long *__restrict__ mass,
+              unsigned *__restrict__ arrived, int *fail) {
+  __shared__ __align__(16) unsigned char sm[kMK * (kMAs + kMBs)];
+  __shared__ int last;
+  if (*bad || (REST && !*need)) return;  // (settled by the kernels before: the same for all blocks)
+  unsigned short *As = (unsigned short *)sm, *Bs = (unsigned short *)(sm + kMK * kMAs);
+  const int first = (nsites + step - 1) / step, total = REST ? nsites - first : first;
+  const int i0 = (int)((int64_t)total * blockIdx.x / gridDim.x), i1 = (int)((int64_t)total * (blockIdx.x + 1) / gridDim.x);
+  const int m0 = blockIdx.y * kMM, j0 = blockIdx.z * kMJ;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int am = threadIdx.x % kMM, ad = threadIdx.x / kMM, bj = threadIdx.x % kMJ, bd = threadIdx.x / kMJ;
+  const bool va = m0 + am < k, vb = j0 + bj < b;
+  const int ea = va ? ev[m0 + am] : 0, eb = vb ? ez[j0 + bj] : 0;
+  const unsigned base = (unsigned)__cvta_generic_to_shared(sm);
+  const unsigned a_addr = base + ((lane >> 4) * 8 + (lane & 7)) * kMAs + ((w & 3) * 16 + (lane >> 3 & 1) * 8) * 2;
+  const unsigned b_addr = base + kMK * kMAs + (lane & 15) * kMBs + (w >> 2) * 16;
+  float c[4] = {0.f, 0.f, 0.f, 0.f};
+  for (int i = i0; i < i1; i += 4) {
+    unsigned a[kMK * kMM / 256], z[kMK * kMJ / 256];
+#pragma unroll
+    for (int u = 0; u < kMK * kMM / 256; ++u) {
+      const int d = ad + u * (256 / kMM), q = i + d / 12;
+      const int64_t s = REST ? q + q / (step - 1) + 1 : (int64_t)q * step;
+      a[u] = q < i1 && va ? mag(Vd[(s * 12 + d % 12) * k + m0 + am], ea) : 0u;
+    }
+#pragma unroll
+    for (int u = 0; u < kMK * kMJ / 256; ++u) {
+      const int d = bd + u * (256 / kMJ), q = i + d / 12;
+      const int64_t s = REST ? q + q / (step - 1) + 1 : (int64_t)q * step;
+      z[u] = q < i1 && vb ? mag(Z[(s * 12 + d % 12) * b + j0 + bj], eb) : 0u;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < kMK * kMM / 256; ++u) As[(ad + u * (256 / kMM)) * (kMAs / 2) + am] = (unsigned short)a[u];
+#pragma unroll
+    for (int u = 0; u < kMK * kMJ / 256; ++u) Bs[(bd + u * (256 / kMJ)) * (kMBs / 2) + bj] = (unsigned short)z[u];
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < kMK / 16; ++q) {
+      unsigned fa[4], b0, b1;
+      ldsm4t(fa, a_addr + q * 16 * kMAs);
+      asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0,%1}, [%2];"
+                   : "=r"(b0), "=r"(b1) : "r"(b_addr + q * 16 * kMBs));
+      mma(c, fa, b0, b1);
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int m = m0 + (w & 3) * 16 + (q >> 1) * 8 + (lane >> 2), j = j0 + (w >> 2) * 8 + (lane & 3) * 2 + (q & 1);
+    if (m < k && j < b && c[q] > 0.f) atomicAdd(&mass[(int64_t)m * b + j], (unsigned long long)(c[q] * 65536.f));
+  }
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(arrived, 1u) == gridDim.x * gridDim.y * gridDim.z - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  int low = 0;
+#pragma unroll 4
+  for (int e = threadIdx.x; e < k * b; e += 256)
+    low |= (float)__ldcg(&mass[e]) < 65536.f * sqrtf(0.5f * (float)count[e % b]);
+  if (__syncthreads_or(low) && threadIdx.x == 0) *fail = 1;
+}
+
 // ------------------------------------------------------------ contraction
 // partial[((chunk * k + m) * 2 + half) * b + j] = sum over the chunk's sites and the half's spins (upper, lower) of
 // conj(V[dof][m]) Z[dof][j].  A block: 32 vectors x 16 columns, one half of the spins, one chunk of sites; stages of 8
@@ -286,7 +391,8 @@ __global__ void __launch_bounds__(256, 2)
 
 // -------------------------------------------------------------- expansion
 // Digit planes of the weights for x0 = V W: Wd[i][2 m + c][2 j + d] as BF16, from W[m][j] 2^ev[m], with rows (Re, Im) of
-// V's entry against columns (Re, Im) of x0: (Wr, Wi; -Wi, Wr); ew[j]: exponent of column j; one block a column.
+// V's entry against columns (Re, Im) of x0: (Wr, Wi; -Wi, Wr); ew[j]: exponent of column j, kZero if it is zero; one
+// block a column.
 __global__ void __launch_bounds__(256) k_oz_weights(const double2 *__restrict__ W, const int *__restrict__ ev, int k,
                                                     int b, unsigned *__restrict__ Wd, int *__restrict__ ew, int *bad) {
   __shared__ int emax, nz;
@@ -303,7 +409,7 @@ __global__ void __launch_bounds__(256) k_oz_weights(const double2 *__restrict__ 
   __syncthreads();
   const int e = nz ? emax : 0;
   if (threadIdx.x == 0) {
-    ew[j] = e;
+    ew[j] = nz ? e : kZero;
     if (e > 800 || e < -800) *bad = 1;  // not finite, or out of the integers' reach
   }
   const int64_t plane = (int64_t)2 * k * b;  // 32-bit pairs of a digit plane
@@ -318,7 +424,8 @@ __global__ void __launch_bounds__(256) k_oz_weights(const double2 *__restrict__ 
   }
 }
 
-// x[dof][j] = sum_m V[dof][m] W[m][j]: a block takes 64 dofs x 16 columns, 32 vectors (64 rows of Wd) a stage
+// x[dof][j] = sum_m V[dof][m] W[m][j]: a block takes 64 dofs x 16 columns, 32 vectors (64 rows of Wd) a stage.
+// *small is set where 16 dofs of a column have squares below `least` in sum (in the weights' units).
 constexpr int kXD = 64, kXM = 32;
 constexpr int kXAs = (2 * kXM + 8) * 2, kXBs = (2 * kOJ + 8) * 2;
 constexpr int kXAp = kXD * kXAs, kXBp = 2 * kXM * kXBs;
@@ -326,7 +433,7 @@ constexpr int kXBytes = kDig * (kXAp + kXBp);
 template <typename VC>
 __global__ void __launch_bounds__(256, 2)
     k_oz_expand(const VC *__restrict__ Vd, const int *__restrict__ ev, const unsigned *__restrict__ Wd,
-                const int *__restrict__ ew, const int *__restrict__ bad, int k, int b, int64_t N,
+                const int *__restrict__ ew, const int *__restrict__ bad, int k, int b, int64_t N, float least, int *small,
                 double2 *__restrict__ x) {
   extern __shared__ __align__(16) unsigned char sm[];
   if (*bad) return;  // the FP64 kernel runs instead
@@ -371,14 +478,23 @@ __global__ void __launch_bounds__(256, 2)
     }
     acc.flush();
 #pragma unroll
-    for (int t = 0; t < 2; ++t)
+    for (int t = 0; t < 2; ++t) {
+      const int j = j0 + ((w >> 2) * 16 + t * 8 + (lane & 3) * 2) / 2;
+      const int e = j < b ? ew[j] : kZero;
+      float sq = 0.f;
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         const int64_t i = i0 + (w & 3) * 16 + h * 8 + (lane >> 2);
-        const int j = j0 + ((w >> 2) * 16 + t * 8 + (lane & 3) * 2) / 2;
-        if (i < N && j < b)
-          x[i * b + j] = make_double2(scalbn(acc.value(t, 2 * h), ew[j]), scalbn(acc.value(t, 2 * h + 1), ew[j]));
+        const double re = acc.value(t, 2 * h), im = acc.value(t, 2 * h + 1);
+        const float fr = f64_to_f32(re), fi = f64_to_f32(im);
+        sq = fmaf(fr, fr, fmaf(fi, fi, sq));
+        if (i < N && j < b) x[i * b + j] = make_double2(scalbn(re, e), scalbn(im, e));
       }
+#pragma unroll
+      for (int o = 4; o < 32; o <<= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+      // (a warp's 16 dofs are all below N or none: N is a multiple of 192)
+      if (sq < least && e != kZero && i0 + (w & 3) * 16 < N) *small = 1;
+    }
   }
 }
 
@@ -394,13 +510,13 @@ int defl_oz_setup(dtr_defl_s *D, cudaStream_t st) {
   const unsigned grid = (unsigned)(8 * device_sms());
   // (an FP32 entry is exact down to 2^-31 of its column's largest; with an exponent of at least -60 subnormals are below)
   if (D->prec == DTR_F64) {
-    k_oz_exp<double2><<<grid, 256, 0, st>>>((const double2 *)D->V, N, k, D->vexp);
+    k_oz_exp<double2><<<grid, 256, 0, st>>>((const double2 *)D->V, N, k, D->vexp, nullptr);
     k_oz_exp_finish<<<4, 256, 0, st>>>(D->vexp, k, 1023, 0x7ff, -800, bad);
   } else {
     if (D->prec == DTR_F32)
-      k_oz_exp<float2><<<grid, 256, 0, st>>>((const float2 *)D->V, N, k, D->vexp);
+      k_oz_exp<float2><<<grid, 256, 0, st>>>((const float2 *)D->V, N, k, D->vexp, nullptr);
     else
-      k_oz_exp<bfc2><<<grid, 256, 0, st>>>((const bfc2 *)D->V, N, k, D->vexp);
+      k_oz_exp<bfc2><<<grid, 256, 0, st>>>((const bfc2 *)D->V, N, k, D->vexp, nullptr);
     k_oz_exp_finish<<<4, 256, 0, st>>>(D->vexp, k, 127, 0xff, -60, bad);
   }
   count_launches(2);
@@ -411,14 +527,47 @@ int defl_oz_setup(dtr_defl_s *D, cudaStream_t st) {
   return DTR_OK;
 }
 
+// scratch in ints: [kBadC] and [kBadX], one pair of flags (the second found while the digits run) that send the
+// contraction or the expansion to the FP64 kernel; [kNeed] the sampled mass fell short, [kArrived] two block counters,
+// [kEz] exponents of Z's columns, [kCount] their nonzero entries, [kEw] exponents of the weights' columns, [kMass] masses
+// (64 bits, k b), behind them the weights' digit planes
+constexpr int kBadC = 0, kBadX = 2, kNeed = 4, kArrived = 5, kEz = 64, kCount = 128, kEw = 192, kMass = 256;
+static size_t planes_at(int k, int b) { return kMass + (size_t)2 * k * b; }
 size_t defl_oz_scratch_bytes(int k, int b) {
-  return 1024 + (size_t)kDig * 2 * k * b * sizeof(unsigned);
+  return (planes_at(k, b) + (size_t)kDig * 2 * k * b) * sizeof(int);
 }
-
-// scratch: [0] bad flag, [64] exponents of Z's columns, [128] of the weights', [256] the weights' digit planes
+const int *defl_oz_contract_flags(const void *scratch) { return (const int *)scratch + kBadC; }
+const int *defl_oz_expand_flags(const void *scratch) { return (const int *)scratch + kBadX; }
 
 template <typename K> static int allow_smem(K kern, int bytes) {
   DTR_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+  return DTR_OK;
+}
+
+// Mass test: on part of the sites first, where Gaussian columns pass with a factor of 4 or more (at 16^3 x 32, k = 64,
+// b = 16 a sixth of them), and on the rest if that falls short.
+template <typename VC> static int mass_t(const dtr_defl_s *D, const double2 *Z, int b, int *sc, cudaStream_t st) {
+  const int V = (int)D->lat.V, k = D->k;
+  int step = (int)(std::sqrt((double)D->lat.N) / 200.0);
+  step = step < 1 ? 1 : step > 64 ? 64 : step;
+  const int tiles = ((k + kMM - 1) / kMM) * ((b + kMJ - 1) / kMJ);
+  auto grid = [&](int sites) {
+    int n = (4 * device_sms() + tiles - 1) / tiles;
+    if (n > (sites + 15) / 16) n = (sites + 15) / 16;
+    return dim3(n < 1 ? 1 : n, (k + kMM - 1) / kMM, (b + kMJ - 1) / kMJ);
+  };
+  unsigned long long *mass = (unsigned long long *)(sc + kMass);
+  k_oz_mass<VC, false><<<grid((V + step - 1) / step), 256, 0, st>>>(
+      (const VC *)D->V, D->vexp, Z, sc + kEz, sc + kCount, sc + kBadC, sc + kNeed, k, b, V, step, mass,
+      (unsigned *)sc + kArrived, sc + (step > 1 ? kNeed : kBadC));
+  count_launches(1);
+  if (step > 1) {
+    k_oz_mass<VC, true><<<grid(V - V / step), 256, 0, st>>>((const VC *)D->V, D->vexp, Z, sc + kEz, sc + kCount, sc + kBadC,
+                                                            sc + kNeed, k, b, V, step, mass, (unsigned *)sc + kArrived + 1,
+                                                            sc + kBadC);
+    count_launches(1);
+  }
+  DTR_LAUNCH_CHECK("digit mass");
   return DTR_OK;
 }
 
@@ -426,10 +575,11 @@ template <typename VC>
 static int contract_t(const dtr_defl_s *D, const double2 *Z, int b, int *sc, int nch, double2 *partial,
                       cudaStream_t st) {
   int rc = allow_smem(k_oz_contract<VC>, kOBytes);
+  if (!rc) rc = mass_t<VC>(D, Z, b, sc, st);
   if (rc) return rc;
   const dim3 grid(2 * nch, (D->k + kOM - 1) / kOM, (b + kOJ - 1) / kOJ);
-  k_oz_contract<VC><<<grid, 256, kOBytes, st>>>((const VC *)D->V, D->vexp, Z, sc + 64, sc, D->k, b, (int)D->lat.V, nch,
-                                               partial);
+  k_oz_contract<VC><<<grid, 256, kOBytes, st>>>((const VC *)D->V, D->vexp, Z, sc + kEz, sc + kBadC, D->k, b,
+                                               (int)D->lat.V, nch, partial);
   count_launches(1);
   return DTR_OK;
 }
@@ -437,9 +587,9 @@ int defl_oz_contract(const dtr_defl_s *D, const double2 *Z, int b, void *scratch
                      int *chunks, cudaStream_t st) {
   int *sc = (int *)scratch;
   const int V = (int)D->lat.V, sms = device_sms();
-  DTR_CUDA(cudaMemsetAsync(sc, 0, 256 * sizeof(int), st));
-  k_oz_exp<double2><<<(unsigned)(8 * sms), 256, 0, st>>>(Z, (int64_t)V * 12, b, sc + 64);
-  k_oz_exp_finish<<<1, 64, 0, st>>>(sc + 64, b, 1023, 0x7ff, -800, sc);
+  DTR_CUDA(cudaMemsetAsync(sc, 0, planes_at(D->k, b) * sizeof(int), st));
+  k_oz_exp<double2><<<(unsigned)(8 * sms), 256, 0, st>>>(Z, (int64_t)V * 12, b, sc + kEz, sc + kCount);
+  k_oz_exp_finish<<<1, 64, 0, st>>>(sc + kEz, b, 1023, 0x7ff, -800, sc + kBadC);
   count_launches(2);
   const int tiles = 2 * ((D->k + kOM - 1) / kOM) * ((b + kOJ - 1) / kOJ);
   int nch = (4 * sms + tiles - 1) / tiles;  // about two rounds of two blocks to an SM
@@ -460,14 +610,17 @@ static int expand_t(const dtr_defl_s *D, int b, int *sc, double2 *x, cudaStream_
   int64_t gx = 2 * device_sms() / nj;
   if (gx < 1) gx = 1;
   if (gx > tiles) gx = tiles;
-  k_oz_expand<VC><<<dim3((unsigned)gx, nj), 256, kXBytes, st>>>((const VC *)D->V, D->vexp, (const unsigned *)(sc + 256),
-                                                                 sc + 128, sc, D->k, b, N, x);
+  const float least = 16.f * (float)D->k * (D->prec == DTR_F64 ? 0x1p-13f : 0x1p-15f);
+  k_oz_expand<VC><<<dim3((unsigned)gx, nj), 256, kXBytes, st>>>((const VC *)D->V, D->vexp,
+                                                                 (const unsigned *)(sc + planes_at(D->k, b)), sc + kEw,
+                                                                 sc + kBadX, D->k, b, N, least, sc + kBadX + 1, x);
   count_launches(1);
   return DTR_OK;
 }
 int defl_oz_expand(const dtr_defl_s *D, const double2 *W, int b, void *scratch, double2 *x, cudaStream_t st) {
   int *sc = (int *)scratch;
-  k_oz_weights<<<b, 256, 0, st>>>(W, D->vexp, D->k, b, (unsigned *)(sc + 256), sc + 128, sc);
+  DTR_CUDA(cudaMemsetAsync(sc + kBadX, 0, 2 * sizeof(int), st));
+  k_oz_weights<<<b, 256, 0, st>>>(W, D->vexp, D->k, b, (unsigned *)(sc + planes_at(D->k, b)), sc + kEw, sc + kBadX);
   count_launches(1);
   if (D->prec == DTR_F64) return expand_t<double2>(D, b, sc, x, st);
   if (D->prec == DTR_F32) return expand_t<float2>(D, b, sc, x, st);
