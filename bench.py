@@ -325,6 +325,18 @@ def run_reference(args):
 
 
 # --------------------------------------------------------------- GPU path
+def shape_that_fits(nbytes, lanes, block, room):
+    """(lanes, block) with nbytes(lanes, block) <= room: the given shape, lanes halved first, then the block."""
+    while nbytes(lanes, block) > room:
+        if lanes > 1:
+            lanes //= 2
+        elif block > 1:
+            block //= 2
+        else:
+            raise MemoryError("one right-hand side needs %d bytes, %d are free" % (nbytes(lanes, block), room))
+    return lanes, block
+
+
 TRAFFIC_F16_B16 = 748.0
 
 
@@ -447,10 +459,10 @@ def main():
     wsh = {"ws": dtr.TraceWorkspace(gauge, defl, params("mixed_f32", L, B, 0, 0, W))}   # current workspace
     base = 1 + rank * 100003
 
-    def step(solver, i, g=None):
+    def step(solver, i, g=None, shape=None):
         run = base + i // steps_per_run
         v0 = (i % steps_per_run) * W
-        return dtr.trace_estimate(g or gauge, w.m0, defl, params(solver, L, B, run, v0, W, GRAPH),
+        return dtr.trace_estimate(g or gauge, w.m0, defl, params(solver, *(shape or (L, B)), run, v0, W, GRAPH),
                                   workspace=wsh["ws"])
 
     # inner-solve storage (FP32 or FP16 Krylov vectors) and cycle driver (one CUDA graph per solve
@@ -522,23 +534,27 @@ def main():
 
     log("32^3x64 mixed", solver=SOLVER, value=value, ms_per_step=total_ms / args.steps, lanes=L, block=B,
         iterations_per_rhs=iters / (args.steps * W), var_T=var_T, trace=[tr_mean.real, tr_mean.imag])
-    # plain FP64 path on the same seeds (the first steps of the timed sequence), in its own workspace
+    # plain FP64 path on the same seeds (the first steps of the timed sequence), in its own workspace; its FP64
+    # vectors take more memory than the mixed solver's, so it may run the same probing vectors in smaller blocks
     wsh["ws"] = None
     torch.cuda.empty_cache()
-    wsh["ws"] = dtr.TraceWorkspace(gauge, defl, params("f64", L, B, 0, 0, W))
+    free, _ = torch.cuda.mem_get_info()
+    shape64 = shape_that_fits(
+        lambda l_, b_: dtr.trace_workspace_bytes(gauge, defl, params("f64", l_, b_, 0, 0, W)), L, B, free - (2 << 30))
+    wsh["ws"] = dtr.TraceWorkspace(gauge, defl, params("f64", *shape64, 0, 0, W))
     ms64, diff = [], 0.0
-    step("f64", 0)                                     # warm-up
+    step("f64", 0, shape=shape64)                      # warm-up
     for i in range(args.f64_steps):
         e0 = torch.cuda.Event(enable_timing=True)
         e1 = torch.cuda.Event(enable_timing=True)
         e0.record()
-        o64 = step("f64", i)
+        o64 = step("f64", i, shape=shape64)
         e1.record()
         torch.cuda.synchronize()
         ms64.append(e0.elapsed_time(e1))
         diff = max(diff, float(np.abs(o64["samples"][0] - samples[i]).max() / np.abs(samples[i]).max()))
     value64 = W * args.f64_steps / (sum(ms64) / 1e3)
-    log("32^3x64 fp64", value=value64, max_rel_sample_diff=diff)
+    log("32^3x64 fp64", value=value64, max_rel_sample_diff=diff, lanes=shape64[0], block=shape64[1])
     wsh["ws"] = None
     torch.cuda.empty_cache()
     wsh["ws"] = dtr.TraceWorkspace(gauge, defl, params("mixed_f32", L, B, 0, 0, W))
@@ -576,6 +592,7 @@ def main():
         "autotune": {"lanes": L, "block": B, "table": [(c["lanes"], c["block"], round(c["rhs_per_s"], 1))
                                                        for c in tune.get("table", [])]},
         "fp64_path": {"value": value64, "unit": UNIT, "steps": args.f64_steps, "ms_per_step": sum(ms64) / len(ms64),
+                      "lanes": shape64[0], "block": shape64[1],
                       "max_rel_sample_diff_vs_mixed": diff},
         "variance_x_time": {"trace": [tr_mean.real, tr_mean.imag], "var_T": var_T, "runs": len(traces),
                             "time_to_1e-3_s": ttr, "time_to_1e-3_s_fp64_path": ttr64,

@@ -587,11 +587,16 @@ def trace_params(seed=0, z0_first=0, n_z0=1, ncolors=1, nvec=1, dilute12=False, 
     return p
 
 
+def trace_workspace_bytes(gauge, defl, params):
+    """Device bytes that trace_estimate needs for these parameters."""
+    return int(_lib.dtr_trace_workspace_bytes(gauge._h, defl._h if defl else None, ctypes.byref(params)))
+
+
 class TraceWorkspace:
     """Reusable device workspace for repeated trace_estimate calls."""
 
     def __init__(self, gauge, defl, params):
-        self.nbytes = _lib.dtr_trace_workspace_bytes(gauge._h, defl._h if defl else None, ctypes.byref(params))
+        self.nbytes = trace_workspace_bytes(gauge, defl, params)
         self.buf = _workspace(self.nbytes)
 
 
