@@ -127,6 +127,25 @@ __global__ void __launch_bounds__(256) unpack_kernel(const typename cplx_t<R>::t
   }
 }
 
+// Blocks of at most kSmallBlock values go one value a thread: the tiles' chain of loads, barrier and stores is longer
+// than all of that takes (an FP32 stencil call, tiles and this: 6x4x10x6 x 3 40.6 and 38.1 us, 8^4 x 2 42.7 and 41.2 us;
+// from 8^4 x 8, 393 k values, on the tiles are as fast, at 8^3 x 16 x 16 56 us against 67).
+constexpr int64_t kSmallBlock = 1 << 18;
+template <typename R>
+__global__ void __launch_bounds__(256) pack_small_kernel(const double2 *__restrict__ canon,
+                                                         typename cplx_t<R>::type *__restrict__ internal, int N, int nrhs,
+                                                         int logb) {
+  typedef typename cplx_t<R>::type C;
+  const int e = blockIdx.x * 256 + threadIdx.x, i = e >> logb, j = e & ((1 << logb) - 1);
+  if (i < N) internal[e] = j < nrhs ? as_c<C>(canon[j * N + i]) : mk<C>(0.0, 0.0);
+}
+template <typename R>
+__global__ void __launch_bounds__(256) unpack_small_kernel(const typename cplx_t<R>::type *__restrict__ internal,
+                                                           double2 *__restrict__ canon, int N, int nrhs, int logb) {
+  const int e = blockIdx.x * 256 + threadIdx.x;
+  if (e < N * nrhs) canon[e] = as_d(internal[((e % N) << logb) + e / N]);
+}
+
 // one column: a plain conversion
 template <typename D, typename S>
 __global__ void __launch_bounds__(256) convert_kernel(const S *__restrict__ in, D *__restrict__ out, int64_t n) {
@@ -148,6 +167,8 @@ void launch_pack(const double2 *canon, typename cplx_t<R>::type *internal, int64
   const int64_t N = V * 12;
   if (b == 1)
     convert_kernel<C, double2><<<tile_grid(N, 8), 256, 0, st>>>(canon, internal, N);
+  else if (N * b <= kSmallBlock)
+    pack_small_kernel<R><<<(unsigned)((N * b + 255) / 256), 256, 0, st>>>(canon, internal, (int)N, nrhs, ilog2(b));
   else
     pack_kernel<R><<<tile_grid(N, b), 256, tile_bytes<C>(b), st>>>(canon, internal, N, nrhs, ilog2(b));
   count_launches(1);
@@ -159,6 +180,8 @@ void launch_unpack(const typename cplx_t<R>::type *internal, double2 *canon, int
   const int64_t N = V * 12;
   if (b == 1)
     convert_kernel<double2, C><<<tile_grid(N, 8), 256, 0, st>>>(internal, canon, N);
+  else if (N * b <= kSmallBlock)
+    unpack_small_kernel<R><<<(unsigned)((N * nrhs + 255) / 256), 256, 0, st>>>(internal, canon, (int)N, nrhs, ilog2(b));
   else
     unpack_kernel<R><<<tile_grid(N, b), 256, tile_bytes<C>(b), st>>>(internal, canon, N, nrhs, ilog2(b));
   count_launches(1);
