@@ -247,7 +247,10 @@ void dtr_solve_params_default(dtr_solve_params *p);
  * z: device, canonical N x nrhs; y: device, canonical N x nrhs, used as the
  * initial guess on entry (zero it for none), solution on exit.  stats: host
  * array of nrhs entries, or NULL.  Returns DTR_ENOTCONV if any RHS missed
- * tol within maxiter (y and stats still written). */
+ * tol within maxiter (y and stats still written).
+ * The persistent engine's BiCGStab solvers run on the red-black Schur complement (sites split by the parity of their
+ * coordinates) unless |4 + m0| < 1/2.  The mixed ones pad a single right-hand side to a pair and take a third more
+ * scratch for it than the whole-lattice ones; in a workspace without that third the whole-lattice ones run. */
 size_t dtr_solve_workspace_bytes(dtr_lattice lat, int nrhs, const dtr_solve_params *p);
 int dtr_solve_batch(dtr_gauge g, double m0, const double *z, double *y, int nrhs,
                     const dtr_solve_params *p, void *work, size_t work_bytes,

@@ -421,11 +421,14 @@ static int check_solve_params(const dtr_solve_params *p) {
   return DTR_OK;
 }
 
+// the solution and right-hand-side blocks of a solve
+static size_t solve_fields_bytes(dtr_lattice lat, int b) {
+  return 256 + 2 * (((size_t)lat->V * 12 * b * sizeof(double2) + 255) / 256 * 256);
+}
 size_t dtr_solve_workspace_bytes(dtr_lattice lat, int nrhs, const dtr_solve_params *p) {
   if (!lat || !p || nrhs < 1 || nrhs > 64) return 0;
   const int b = pad_rhs(nrhs);
-  const size_t vb = ((size_t)lat->V * 12 * b * sizeof(double2) + 255) / 256 * 256;
-  return 256 + 2 * vb + solver_scratch_bytes(lat->V, b, p->solver, p->gmres_m);
+  return solve_fields_bytes(lat, b) + solver_scratch_bytes(lat->V, b, p->solver, p->gmres_m);
 }
 
 int dtr_solve_batch(dtr_gauge g, double m0, const double *z, double *y, int nrhs, const dtr_solve_params *p,
@@ -434,10 +437,10 @@ int dtr_solve_batch(dtr_gauge g, double m0, const double *z, double *y, int nrhs
   if (nrhs < 1 || nrhs > 64) return fail(DTR_EINVAL, "nrhs must be in [1, 64]");
   int rc = check_solve_params(p);
   if (rc) return rc;
-  const size_t need = dtr_solve_workspace_bytes(&g->lat, nrhs, p);
-  if (work_bytes < need) return fail(DTR_ENOMEM, "solver workspace too small");
-  cudaStream_t st = (cudaStream_t)stream;
   const int b = pad_rhs(nrhs);
+  if (work_bytes < solve_fields_bytes(&g->lat, b) + solver_scratch_least(g->lat.V, b, p->solver, p->gmres_m))
+    return fail(DTR_ENOMEM, "solver workspace too small");
+  cudaStream_t st = (cudaStream_t)stream;
   const size_t vb = ((size_t)g->lat.V * 12 * b * sizeof(double2) + 255) / 256 * 256;
   char *w = (char *)(((uintptr_t)work + 255) & ~(uintptr_t)255);
   double2 *X = (double2 *)w, *Z = (double2 *)(w + vb);

@@ -532,7 +532,7 @@ __global__ void k_scal_init(Scal *sc, int b, double tol2, int maxiter) {
     sc->flags[j] = 0;
     sc->rho[j] = sc->alpha[j] = sc->omega[j] = sc->beta[j] = make_double2(0.0, 0.0);
     sc->rnorm2[j] = sc->bnorm2[j] = sc->rtrue2[j] = 0.0;
-    sc->scale[j] = sc->base[j] = sc->fac[j] = 1.0;
+    sc->scale[j] = 1.0;
   }
   if (j == 0) {
     sc->n_active = 0;
@@ -618,18 +618,26 @@ static double inner_tol_for(const dtr_solve_params *p) {
   return t < floor ? floor : t;
 }
 
-size_t solver_scratch_bytes(int64_t V, int b, int solver, int gmres_m) {
+size_t solver_scratch_least(int64_t V, int b, int solver, int gmres_m) {
   const size_t vec64 = ((size_t)V * 12 * b * sizeof(double2) + 255) / 256 * 256;
   const size_t vec32 = ((size_t)V * 12 * b * sizeof(float2) + 255) / 256 * 256;
   const size_t red = 256 + (size_t)kMaxGrid * 5 * 64 * sizeof(double2);
   const size_t scal = 2 * ((sizeof(Scal) + 255) / 256) * 256;
   const size_t fixed = 256 + red + scal + 256 + 256;
-  if (mixed_bicgstab(solver)) {  // half storage uses half of each slot; the larger of the two cycles' buffers
-    const size_t full = vec64 + 7 * vec32, eo = eo_scratch_bytes(V, b);
-    return fixed + (full > eo ? full : eo);
-  }
+  if (mixed_bicgstab(solver)) return fixed + vec64 + 7 * vec32;  // half storage uses half of each slot
   if (solver == DTR_SOLVER_FGMRES_NET) return fixed + vec64 + 7 * vec32 + fgmres_scratch_bytes(V, b, gmres_m) + 256;
   return fixed + 6 * vec64;
+}
+
+// what the red-black cycles take beyond the whole-lattice ones: 6 half-lattice vectors for one column, else nothing
+static size_t eo_extra_bytes(int64_t V, int b) {
+  const size_t full = ((size_t)V * 12 * b * sizeof(double2) + 255) / 256 * 256 +
+                      7 * (((size_t)V * 12 * b * sizeof(float2) + 255) / 256 * 256);
+  const size_t eo = eo_scratch_bytes(V, b);
+  return eo > full ? eo - full : 0;
+}
+size_t solver_scratch_bytes(int64_t V, int b, int solver, int gmres_m) {
+  return solver_scratch_least(V, b, solver, gmres_m) + (mixed_bicgstab(solver) ? eo_extra_bytes(V, b) : 0);
 }
 
 static char *align256(char *p) { return (char *)(((uintptr_t)p + 255) & ~(uintptr_t)255); }
@@ -1057,7 +1065,7 @@ int solve_internal(const dtr_gauge_s *gauge, double m0, double2 *x, const double
                    int x_is_zero, int async) {
   const Geom g = geom_of(gauge->lat);
   const int64_t n = (int64_t)g.V * 12 * b;
-  if (work_bytes < solver_scratch_bytes(g.V, b, p->solver, p->gmres_m))
+  if (work_bytes < solver_scratch_least(g.V, b, p->solver, p->gmres_m))
     return fail(DTR_ENOMEM, "solver workspace too small");
   char *w = align256((char *)work);
   Reduce red;
@@ -1092,7 +1100,8 @@ int solve_internal(const dtr_gauge_s *gauge, double m0, double2 *x, const double
   S.store = store;
   S.hs = hs;
   S.upd = resid_update_enabled(store) ? 1 : 0;
-  S.eo = mixed_bicgstab(p->solver) && persistent && eo_usable(m0);
+  S.eo = mixed_bicgstab(p->solver) && persistent && eo_usable(m0) &&
+         work_bytes >= solver_scratch_bytes(g.V, b, p->solver, p->gmres_m);
   if (mixed_bicgstab(p->solver) && persistent && !p->no_graph) {
     carve_mixed(S, w);
     *scal_out = outer;

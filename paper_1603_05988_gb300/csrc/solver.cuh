@@ -13,10 +13,14 @@ constexpr double kInnerTolFloorBF16 = 1e-2;  // and of BF16-stored ones
 
 // Per-column Krylov scalars, resident in device memory (b <= 64 columns).
 struct Scal {
-  double2 rho[64], alpha[64], omega[64], beta[64];
+  double2 rho[64], alpha[64], omega[64];
+  union {
+    double2 beta[64];
+    struct {
+      double base[64], fac[64];  // red-black defect correction, which has no recursion of its own: powers of two that
+    };                           // scale the residual as it is kept, and that to the inner right-hand side (0: column
+  };                             // not iterated)
   double rnorm2[64], bnorm2[64], rtrue2[64], scale[64];
-  double base[64], fac[64];  // red-black defect correction: powers of two that scale the residual as it is kept, and
-                             // that to the inner right-hand side (0: column not iterated)
   int active[64], iters[64], restarts[64], conv[64], flags[64];
   int n_active;
   int maxiter;
@@ -27,8 +31,10 @@ template <typename R> struct KrylovVecs {
   typename cplx_t<R>::type *x, *r, *rhat, *p, *v, *t;
 };
 
-// Scratch the solver needs beyond the solution and right-hand-side blocks.
+// Scratch the solver takes beyond the solution and right-hand-side blocks, and the least it runs in: the red-black
+// mixed solvers pad a single column to a pair, and in a workspace too small for that the whole-lattice ones run.
 size_t solver_scratch_bytes(int64_t V, int b, int solver, int gmres_m = 16);
+size_t solver_scratch_least(int64_t V, int b, int solver, int gmres_m = 16);
 
 // Solve A x = z on internal-layout FP64 blocks of width b.  x holds the
 // initial guess on entry.  *scal receives the device pointer of the final

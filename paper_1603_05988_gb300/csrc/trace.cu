@@ -188,13 +188,15 @@ static int trace_lanes(const dtr_trace_params *p) {
   return l;
 }
 
-static TraceLayout trace_layout(const dtr_gauge_s *g, const dtr_defl_s *D, const dtr_trace_params *p) {
+// least: the smallest workspace that the solver runs in
+static TraceLayout trace_layout(const dtr_gauge_s *g, const dtr_defl_s *D, const dtr_trace_params *p,
+                                bool least = false) {
   TraceLayout L;
   L.b = pad_rhs(p->block);
   const int64_t V = g->lat.V;
   L.vec = al((size_t)V * 12 * L.b * sizeof(double2));
   L.zdot_red = al(256 + (size_t)kMaxGrid * 64 * sizeof(double2));
-  L.solver = al(solver_scratch_bytes(V, L.b, p->solve.solver, p->solve.gmres_m));
+  L.solver = al((least ? solver_scratch_least : solver_scratch_bytes)(V, L.b, p->solve.solver, p->solve.gmres_m));
   L.defl = D ? al(defl_scratch_bytes(V, D->k, L.b, device_sms())) : 0;
   const bool hp = D && p->ncolors > 1;
   L.hp = hp ? al(defl_hp_scratch_bytes(V, D->k, L.b, p->ncolors, device_sms())) : 0;
@@ -213,6 +215,9 @@ static TraceLayout trace_layout(const dtr_gauge_s *g, const dtr_defl_s *D, const
 
 size_t trace_workspace_bytes(const dtr_gauge_s *g, const dtr_defl_s *D, const dtr_trace_params *p) {
   return trace_layout(g, D, p).total;
+}
+size_t trace_workspace_least(const dtr_gauge_s *g, const dtr_defl_s *D, const dtr_trace_params *p) {
+  return trace_layout(g, D, p, true).total;
 }
 
 // Per-lane device buffers, stream and pinned host staging.
@@ -263,7 +268,8 @@ static int lane_host_buffers(int l, int k) {
 
 int trace_estimate(const dtr_gauge_s *gauge, double m0, const dtr_defl_s *D, const dtr_trace_params *p, void *work,
                    size_t work_bytes, dtr_trace_result *res, cudaStream_t st) {
-  const TraceLayout L = trace_layout(gauge, D, p);
+  TraceLayout L = trace_layout(gauge, D, p);
+  if (work_bytes < L.total) L = trace_layout(gauge, D, p, true);
   if (work_bytes < L.total) return fail(DTR_ENOMEM, "trace workspace too small");
   const int b = L.b;
   const Geom g = geom_of(gauge->lat);

@@ -23,6 +23,7 @@ namespace dtr {
 int trace_estimate(const dtr_gauge_s *gauge, double m0, const dtr_defl_s *D, const dtr_trace_params *p, void *work,
                    size_t work_bytes, dtr_trace_result *res, cudaStream_t st);
 size_t trace_workspace_bytes(const dtr_gauge_s *g, const dtr_defl_s *D, const dtr_trace_params *p);
+size_t trace_workspace_least(const dtr_gauge_s *g, const dtr_defl_s *D, const dtr_trace_params *p);
 
 namespace {
 
@@ -124,7 +125,7 @@ int trace_autotune(const dtr_gauge_s *g, double m0, const dtr_defl_s *D, const d
   for (int blk : blocks) {
     for (int lanes : kLaneCands) {
       const dtr_trace_params q = candidate(p, lanes, blk);
-      const size_t need = trace_workspace_bytes(g, D, &q);
+      const size_t need = trace_workspace_least(g, D, &q);
       if (need > work_bytes) continue;
       dtr_trace_result r;
       std::memset(&r, 0, sizeof(r));
