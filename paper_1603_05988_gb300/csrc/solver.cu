@@ -629,7 +629,16 @@ size_t solver_scratch_least(int64_t V, int b, int solver, int gmres_m) {
   return fixed + 6 * vec64;
 }
 
-// what the red-black cycles take beyond the whole-lattice ones: 6 half-lattice vectors for one column, else nothing
+// Red-black cycles pay.  A single column is padded to a pair and a Schur application reads every link twice, so that on
+// large lattices the whole-lattice solver is faster for it (us a solve, red-black and whole lattice, eps 0.8 and 0.5):
+// FP32 24^3 x 48 14410, 15420 and 17930, 19080; 32^4 24510, 22710 and 28720, 29100; 32^3 x 64 48440, 43660 and 56840, 54420
+// FP16 20^3 x 32  5910,  6570 and  6700,  7050; 24^3 x 32 9470, 8820 and 10800, 10300
+// BF16 12^4       1380,  1870 and  1570,  2420; 16^4 2370, 2160 and 2700, 2580; 16^3 x 32 4090, 3500 and 4820, 4080
+// From two columns on red-black is faster at every size (BF16 at 32^3 x 64: 54200 against 62900).
+static bool eo_pays(int64_t V, int b, int store) {
+  return b > 1 || V < (store == 0 ? 1 << 20 : store == 1 ? 3 << 17 : 1 << 16);
+}
+// what they take beyond the whole-lattice ones: 6 half-lattice vectors for one column, else nothing
 static size_t eo_extra_bytes(int64_t V, int b) {
   const size_t full = ((size_t)V * 12 * b * sizeof(double2) + 255) / 256 * 256 +
                       7 * (((size_t)V * 12 * b * sizeof(float2) + 255) / 256 * 256);
@@ -637,7 +646,8 @@ static size_t eo_extra_bytes(int64_t V, int b) {
   return eo > full ? eo - full : 0;
 }
 size_t solver_scratch_bytes(int64_t V, int b, int solver, int gmres_m) {
-  return solver_scratch_least(V, b, solver, gmres_m) + (mixed_bicgstab(solver) ? eo_extra_bytes(V, b) : 0);
+  const bool eo = mixed_bicgstab(solver) && eo_pays(V, b, inner_store(solver));
+  return solver_scratch_least(V, b, solver, gmres_m) + (eo ? eo_extra_bytes(V, b) : 0);
 }
 
 static char *align256(char *p) { return (char *)(((uintptr_t)p + 255) & ~(uintptr_t)255); }
@@ -1100,7 +1110,7 @@ int solve_internal(const dtr_gauge_s *gauge, double m0, double2 *x, const double
   S.store = store;
   S.hs = hs;
   S.upd = resid_update_enabled(store) ? 1 : 0;
-  S.eo = mixed_bicgstab(p->solver) && persistent && eo_usable(m0) &&
+  S.eo = mixed_bicgstab(p->solver) && persistent && eo_usable(m0) && eo_pays(g.V, b, store) &&
          work_bytes >= solver_scratch_bytes(g.V, b, p->solver, p->gmres_m);
   if (mixed_bicgstab(p->solver) && persistent && !p->no_graph) {
     carve_mixed(S, w);
