@@ -368,7 +368,8 @@ int dtr_defl_to_host(dtr_defl d, double *V_host, double *lambda_host);
  * Accuracy: that of FP64 sums, C to about 2^-53 of sum |v| |z|.  Larger blocks run on the tensor cores in integers
  * relative to each column's largest entry, with 54 bits; blocks for which that would lose digits (entries small in V
  * where z is large or the other way round, point sources, solutions x0 that are small over a whole neighbourhood of 16
- * dofs; not finite values) are found on the device and take FP64 sums, at the FP64 pipe's rate.
+ * dofs; not finite values) are found on the device and take FP64 sums, at the FP64 pipe's rate.  So does a workspace
+ * without the integers' share of it, 64 k nrhs bytes and some (nrhs rounded up to a power of two).
  * work: device workspace of dtr_deflate_workspace_bytes(d, nrhs) bytes. */
 size_t dtr_deflate_workspace_bytes(dtr_defl d, int nrhs);
 int dtr_deflate_project(dtr_defl d, const double *z, int nrhs, double *d_out, double *coeff_out,

@@ -673,20 +673,25 @@ int dtr_defl_gram(dtr_defl d, dtr_gauge g, double m0, void *stream) {
   return defl_gram(d, g, m0, (cudaStream_t)stream);
 }
 
+// the blocks and coefficients of a projection
+static size_t deflate_fields_bytes(dtr_defl d, int b) {
+  const size_t vb = ((size_t)d->lat.V * 12 * b * sizeof(double2) + 255) / 256 * 256;
+  return 256 + 2 * vb + 256 * 3 + 64 * sizeof(double2);
+}
 size_t dtr_deflate_workspace_bytes(dtr_defl d, int nrhs) {
   if (!d || nrhs < 1 || nrhs > 64) return 0;
   const int b = pad_rhs(nrhs);
-  const size_t vb = ((size_t)d->lat.V * 12 * b * sizeof(double2) + 255) / 256 * 256;
-  return 256 + 2 * vb + 256 * 3 + 64 * sizeof(double2) + defl_scratch_bytes(d->lat.V, d->k, b, device_sms());
+  return deflate_fields_bytes(d, b) + defl_scratch_bytes(d->lat.V, d->k, b, device_sms());
 }
 
 int dtr_deflate_project(dtr_defl d, const double *z, int nrhs, double *d_out, double *coeff_out, double *x0_out,
                         void *work, size_t work_bytes, void *stream) {
   if (!d || !z || !d_out || !work) return fail(DTR_EINVAL, "null argument");
   if (nrhs < 1 || nrhs > 64) return fail(DTR_EINVAL, "nrhs must be in [1, 64]");
-  if (work_bytes < dtr_deflate_workspace_bytes(d, nrhs)) return fail(DTR_ENOMEM, "deflation workspace too small");
-  cudaStream_t st = (cudaStream_t)stream;
   const int b = pad_rhs(nrhs);
+  if (work_bytes < deflate_fields_bytes(d, b) + defl_scratch_least(d->lat.V, d->k, b, device_sms()))
+    return fail(DTR_ENOMEM, "deflation workspace too small");
+  cudaStream_t st = (cudaStream_t)stream;
   const size_t vb = ((size_t)d->lat.V * 12 * b * sizeof(double2) + 255) / 256 * 256;
   char *w = (char *)(((uintptr_t)work + 255) & ~(uintptr_t)255);
   double2 *Z = (double2 *)w;
@@ -873,26 +878,31 @@ int dtr_trace_estimate(dtr_gauge g, double m0, dtr_defl d, const dtr_trace_param
   return trace_estimate(g, m0, d, p, work, work_bytes, res, (cudaStream_t)stream);
 }
 
+// all but the projection's scratch
+static size_t time_deflate_fields_bytes(dtr_defl d, int b) {
+  return (((size_t)d->lat.V * 12 * b * sizeof(double2) + 255) / 256) * 256 + 64 * sizeof(double2) + 256 + 256 +
+         (((size_t)d->lat.V * 12 * b + 255) / 256) * 256;
+}
 size_t dtr_time_deflate_workspace_bytes(dtr_defl d, int nrhs) {
   if (!d || nrhs < 1 || nrhs > 64) return 0;
   const int b = pad_rhs(nrhs);
-  return (((size_t)d->lat.V * 12 * b * sizeof(double2) + 255) / 256) * 256 + 64 * sizeof(double2) + 256 +
-         defl_scratch_bytes(d->lat.V, d->k, b, device_sms()) + 256 + (((size_t)d->lat.V * 12 * b + 255) / 256) * 256;
+  return time_deflate_fields_bytes(d, b) + defl_scratch_bytes(d->lat.V, d->k, b, device_sms());
 }
 
 int dtr_time_deflate(dtr_defl d, int nrhs, int reps, void *work, size_t work_bytes, double *avg_ms, void *stream) {
   if (!d || !work || !avg_ms) return fail(DTR_EINVAL, "null argument");
   if (nrhs < 1 || nrhs > 64 || reps < 1) return fail(DTR_EINVAL, "nrhs must be in [1, 64] and reps >= 1");
-  if (work_bytes < dtr_time_deflate_workspace_bytes(d, nrhs)) return fail(DTR_ENOMEM, "workspace too small");
-  cudaStream_t st = (cudaStream_t)stream;
   const int b = pad_rhs(nrhs);
+  size_t sb = defl_scratch_bytes(d->lat.V, d->k, b, device_sms());
+  if (work_bytes < time_deflate_fields_bytes(d, b) + sb) sb = defl_scratch_least(d->lat.V, d->k, b, device_sms());
+  if (work_bytes < time_deflate_fields_bytes(d, b) + sb) return fail(DTR_ENOMEM, "workspace too small");
+  cudaStream_t st = (cudaStream_t)stream;
   const Geom geo = geom_of(d->lat);
   char *w = (char *)(((uintptr_t)work + 255) & ~(uintptr_t)255);
   double2 *Z = (double2 *)w;
   w += (((size_t)d->lat.V * 12 * b * sizeof(double2) + 255) / 256) * 256;
   double2 *dd = (double2 *)w;
   w += 64 * sizeof(double2) + 256;
-  const size_t sb = defl_scratch_bytes(d->lat.V, d->k, b, device_sms());
   unsigned char *Zc = (unsigned char *)(w + ((sb + 255) / 256) * 256);  // the block as one-byte codes
   launch_noise(Z, geo, 0x5EED, 0, 1, 0, 0, 1, nrhs, b, st, 0, Zc);  // one Z4 vector per column
   int rc = defl_project_internal(d, Z, b, dd, nullptr, nullptr, nullptr, w, sb, device_sms(), st, 1, Zc);  // warm

@@ -325,15 +325,18 @@ static int defl_chunks(int64_t V, int k, int b, int sms) {
   return (int)want;
 }
 
-size_t defl_scratch_bytes(int64_t V, int k, int b, int sms) {
+size_t defl_scratch_least(int64_t V, int k, int b, int sms) {
   const int nch = defl_chunks(V, k, b, sms);
   size_t part = (size_t)nch * k * 2 * b * sizeof(double2);
   const size_t tc = defl_tc_scratch_bytes(V, k, b, sms);  // the tensor-core partials share this region
   if (tc > part) part = tc;
   const size_t C = (size_t)k * 2 * b * sizeof(double2);
   const size_t W = (size_t)k * b * sizeof(double2);
-  const size_t d = 64 * sizeof(double2) + defl_oz_scratch_bytes(k, b) + 256;
+  const size_t d = 64 * sizeof(double2);
   return ((part + 255) / 256 + (C + 255) / 256 + (W + 255) / 256 + (d + 255) / 256 + 5) * 256;
+}
+size_t defl_scratch_bytes(int64_t V, int k, int b, int sms) {
+  return defl_scratch_least(V, k, b, sms) + (defl_oz_scratch_bytes(k, b) + 255) / 256 * 256;
 }
 
 // layout of the scratch: [status word, 256 B][partials][C][x0 weights]
@@ -352,7 +355,8 @@ int defl_project_internal(const dtr_defl_s *D, const double2 *Z, int b, double2 
                           cudaStream_t st, int z4, const unsigned char *Zc) {
   const int64_t V = D->lat.V;
   const int k = D->k;
-  if (work_bytes < defl_scratch_bytes(V, k, b, sms)) return fail(DTR_ENOMEM, "deflation workspace too small");
+  if (work_bytes < defl_scratch_least(V, k, b, sms)) return fail(DTR_ENOMEM, "deflation workspace too small");
+  const bool digits = D->vexp_ok && work_bytes >= defl_scratch_bytes(V, k, b, sms);
   const int nch = defl_chunks(V, k, b, sms);
   const int G = kDeflBlock / b;
   const int tiles = (k + G * kMPT - 1) / (G * kMPT);
@@ -379,7 +383,7 @@ int defl_project_internal(const dtr_defl_s *D, const double2 *Z, int b, double2 
     // digits on the tensor cores; what is beyond them (found on the device) the FP64 kernel does, on the same chunks
     int chunks = nch;
     const int *bad = nullptr;
-    if (D->vexp_ok && oz_contract_pays(V)) {
+    if (digits && oz_contract_pays(V)) {
       int rc = defl_oz_contract(D, Z, b, oz, nch, partial, &chunks, st);
       if (rc) return rc;
       bad = defl_oz_contract_flags(oz);
@@ -404,7 +408,7 @@ int defl_project_internal(const dtr_defl_s *D, const double2 *Z, int b, double2 
     unsigned grid = (unsigned)((n + 255) / 256);
     if (grid > 16u * (unsigned)sms) grid = 16u * (unsigned)sms;
     const int *bad = nullptr;
-    if (D->vexp_ok && oz_expand_pays(V * 12, k, b)) {
+    if (digits && oz_expand_pays(V * 12, k, b)) {
       int rc = defl_oz_expand(D, Wx, b, oz, x0_internal, st);
       if (rc) return rc;
       bad = defl_oz_expand_flags(oz);

@@ -17,6 +17,8 @@ __device__ __forceinline__ double2 vload(const bfc2 &v) { return f32_to_f64(__bf
 
 // Scratch for one projection of a width-b block.
 size_t defl_scratch_bytes(int64_t V, int k, int b, int sms);  // includes k x b expansion weights
+// The least it runs in: without the tensor-core digits of general blocks (deflate_oz.cu).
+size_t defl_scratch_least(int64_t V, int k, int b, int sms);
 
 // C = V^H [Z, g5 Z] (k x 2b, kept in scratch; *C_out points at it),
 // d_dev[j] = sum_m conj(C[m,j]) C[m,b+j] / lambda_m, terms_dev (k x b, or

@@ -188,7 +188,7 @@ static int trace_lanes(const dtr_trace_params *p) {
   return l;
 }
 
-// least: the smallest workspace that the solver runs in
+// least: the smallest workspace that the solver and the projection run in
 static TraceLayout trace_layout(const dtr_gauge_s *g, const dtr_defl_s *D, const dtr_trace_params *p,
                                 bool least = false) {
   TraceLayout L;
@@ -197,7 +197,7 @@ static TraceLayout trace_layout(const dtr_gauge_s *g, const dtr_defl_s *D, const
   L.vec = al((size_t)V * 12 * L.b * sizeof(double2));
   L.zdot_red = al(256 + (size_t)kMaxGrid * 64 * sizeof(double2));
   L.solver = al((least ? solver_scratch_least : solver_scratch_bytes)(V, L.b, p->solve.solver, p->solve.gmres_m));
-  L.defl = D ? al(defl_scratch_bytes(V, D->k, L.b, device_sms())) : 0;
+  L.defl = D ? al((least ? defl_scratch_least : defl_scratch_bytes)(V, D->k, L.b, device_sms())) : 0;
   const bool hp = D && p->ncolors > 1;
   L.hp = hp ? al(defl_hp_scratch_bytes(V, D->k, L.b, p->ncolors, device_sms())) : 0;
   L.sites = hp ? al((size_t)V * sizeof(int)) : 0;
