@@ -905,6 +905,7 @@ int dtr_time_deflate(dtr_defl d, int nrhs, int reps, void *work, size_t work_byt
   w += 64 * sizeof(double2) + 256;
   unsigned char *Zc = (unsigned char *)(w + ((sb + 255) / 256) * 256);  // the block as one-byte codes
   launch_noise(Z, geo, 0x5EED, 0, 1, 0, 0, 1, nrhs, b, st, 0, Zc);  // one Z4 vector per column
+  DTR_CUDA(cudaMemsetAsync(defl_error_word(w), 0, sizeof(int), st));  // only the tensor-core contraction sets it
   int rc = defl_project_internal(d, Z, b, dd, nullptr, nullptr, nullptr, w, sb, device_sms(), st, 1, Zc);  // warm
   if (rc) return rc;
   cudaEvent_t e0, e1;
