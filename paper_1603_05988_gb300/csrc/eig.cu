@@ -451,7 +451,8 @@ static int eig_basis_size(const dtr_eig_params *P) {
   return (p + 15) / 16 * 16;
 }
 
-static EigLayout eig_layout(const dtr_lattice_s &lat, const dtr_eig_params *P) {
+// least: with as few Gram chunks as the FP32 tiles take, the smallest workspace that it runs in
+static EigLayout eig_layout(const dtr_lattice_s &lat, const dtr_eig_params *P, bool least = false) {
   EigLayout L;
   L.p = eig_basis_size(P);
   L.b = P->chunk > 0 ? pad_rhs(P->chunk) : 32;
@@ -460,11 +461,12 @@ static EigLayout eig_layout(const dtr_lattice_s &lat, const dtr_eig_params *P) {
   const size_t cs = P->store == DTR_F64 ? 16 : 8;  // chunk fields: FP64 or FP32 arithmetic
   // dof chunks of a Gram product: enough blocks for four to an SM, each with a run of dofs long enough to outweigh
   // its partial sums (16-wide FP64 tiles take 16 dofs in as many FP64 instructions as their sums take loads)
-  const int GT = P->store == DTR_F64 ? 16 * gram_rt<double2>() : kGT;
+  const bool small_tiles = P->store == DTR_F64 && !least;
+  const int GT = small_tiles ? 16 * gram_rt<double2>() : kGT;
   const int tiles = ((L.p + GT - 1) / GT) * ((L.p + GT - 1) / GT);
-  const int run = P->store == DTR_F64 ? 256 : 4096;
+  const int run = small_tiles ? 256 : 4096;
   int64_t nk = (4LL * device_sms() + tiles - 1) / tiles;
-  if (P->store == DTR_F64 && nk < 8) nk = 8;
+  if (small_tiles && nk < 8) nk = 8;
   const int64_t maxk = N / run > 0 ? N / run : 1;
   if (nk > maxk) nk = maxk;
   if (nk < 1) nk = 1;
@@ -619,7 +621,8 @@ static int eig_solve_t(const dtr_gauge_s *gauge, double m0, const dtr_eig_params
                        dtr_defl_s *D, double *res_out, dtr_eig_stats *stats, cudaStream_t st) {
   typedef typename EigAcc<T>::type AC;
   const auto t_start = std::chrono::steady_clock::now();
-  const EigLayout L = eig_layout(gauge->lat, P);
+  EigLayout L = eig_layout(gauge->lat, P);
+  if (work_bytes < L.total) L = eig_layout(gauge->lat, P, true);
   if (work_bytes < L.total) return fail(DTR_ENOMEM, "eigensolver workspace too small");
   const int64_t N = gauge->lat.N;
   const int p = L.p, k = P->k, b = L.b;
