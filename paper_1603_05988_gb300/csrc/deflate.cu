@@ -66,9 +66,12 @@ __global__ void __launch_bounds__(kDeflBlock)
   }
 }
 
-// C (column-major k x 2b): C[m + k*j] = P + Q, C[m + k*(b+j)] = P - Q
-__global__ void k_defl_reduce(const double2 *__restrict__ partial, int k, int b, int nchunks, double2 *__restrict__ C) {
+// C (column-major k x 2b): C[m + k*j] = P + Q, C[m + k*(b+j)] = P - Q.  With flags that are not set the digits wrote the
+// partial sums, over their own number of chunks.
+__global__ void k_defl_reduce(const double2 *__restrict__ partial, int k, int b, int nchunks, const int *flags,
+                              int digit_chunks, double2 *__restrict__ C) {
   const int64_t n = (int64_t)k * b;
+  if (flags && !(flags[0] | flags[1])) nchunks = digit_chunks;
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
     const int j = (int)(e % b);
     const int m = (int)(e / b);
@@ -380,8 +383,9 @@ int defl_project_internal(const dtr_defl_s *D, const double2 *Z, int b, double2 
     int rc = defl_contract_tc(D, Z, b, C, partial, partbytes, err, sms, st, Zc);
     if (rc) return rc;
   } else {
-    // digits on the tensor cores; what is beyond them (found on the device) the FP64 kernel does, on the same chunks
-    int chunks = nch;
+    // digits on the tensor cores; what is beyond them (found on the device) the FP64 kernel does, on chunks of its own (on
+    // the digits' 16, point sources at 4^4 in an FP64 space with k = 8 and x0 took 324 us, 204 us so)
+    int chunks = 0;
     const int *bad = nullptr;
     if (digits && oz_contract_pays(V)) {
       int rc = defl_oz_contract(D, Z, b, oz, nch, partial, &chunks, st);
@@ -389,15 +393,15 @@ int defl_project_internal(const dtr_defl_s *D, const double2 *Z, int b, double2 
       bad = defl_oz_contract_flags(oz);
     }
     if (D->prec == DTR_F64)
-      k_defl_partial<double2><<<chunks * tiles, kDeflBlock, 0, st>>>((const double2 *)D->V, Z, k, b, logb, (int)V, chunks,
-                                                                     partial, bad);
-    else if (D->prec == DTR_F32)
-      k_defl_partial<float2><<<chunks * tiles, kDeflBlock, 0, st>>>((const float2 *)D->V, Z, k, b, logb, (int)V, chunks,
-                                                                    partial, bad);
-    else
-      k_defl_partial<bfc2><<<chunks * tiles, kDeflBlock, 0, st>>>((const bfc2 *)D->V, Z, k, b, logb, (int)V, chunks,
+      k_defl_partial<double2><<<nch * tiles, kDeflBlock, 0, st>>>((const double2 *)D->V, Z, k, b, logb, (int)V, nch,
                                                                   partial, bad);
-    k_defl_reduce<<<(unsigned)((nkb + 255) / 256), 256, 0, st>>>(partial, k, b, chunks, C);
+    else if (D->prec == DTR_F32)
+      k_defl_partial<float2><<<nch * tiles, kDeflBlock, 0, st>>>((const float2 *)D->V, Z, k, b, logb, (int)V, nch,
+                                                                 partial, bad);
+    else
+      k_defl_partial<bfc2><<<nch * tiles, kDeflBlock, 0, st>>>((const bfc2 *)D->V, Z, k, b, logb, (int)V, nch, partial,
+                                                               bad);
+    k_defl_reduce<<<(unsigned)((nkb + 255) / 256), 256, 0, st>>>(partial, k, b, nch, bad, chunks, C);
     count_launches(2);
   }
   if (d_dev) launch_defl_d(D, C, b, d_dev, terms_dev, st);
