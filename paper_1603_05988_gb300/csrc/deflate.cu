@@ -438,6 +438,7 @@ int defl_trace_TD(dtr_defl_s *D, cudaStream_t st) {
   if (nch64 > nsite) nch64 = nsite;
   const int nch = (int)nch64;
   double *part = nullptr, *td = nullptr;
+  D->vexp_ok = false;
   DTR_CUDA(cudaMalloc((void **)&part, (size_t)nch * k * sizeof(double) + 256));
   td = (double *)((char *)part + (((size_t)nch * k * sizeof(double) + 127) / 128) * 128);
   const dim3 grid(nch, mt);
@@ -449,15 +450,22 @@ int defl_trace_TD(dtr_defl_s *D, cudaStream_t st) {
     k_defl_td_partial<bfc2><<<grid, kTdThreads, 0, st>>>((const bfc2 *)D->V, k, nsite, nch, part);
   count_launches(1);
   k_defl_td_reduce<<<1, kTdThreads, 0, st>>>(part, D->inv_lambda, k, nch, td); count_launches(1);
+  // the digits' exponents, waited for together with T_D
+  const int rc = defl_oz_setup(D, (int *)(td + 1), st);
   cudaError_t e = cudaGetLastError();
-  double h = 0.0;
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&h, td, sizeof(double), cudaMemcpyDeviceToHost, st);
+  struct {
+    double td;
+    int bad, pad;
+  } h = {0.0, 1, 0};
+  if (e == cudaSuccess) e = cudaMemcpyAsync(&h, td, sizeof(h), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   cudaFree(part);
+  if (rc) return rc;
   if (e != cudaSuccess) return cuda_fail(e, "T_D reduction");
-  D->td[0] = h;
+  D->td[0] = h.td;
   D->td[1] = 0.0;
-  return defl_oz_setup(D, st);
+  D->vexp_ok = h.bad == 0;
+  return DTR_OK;
 }
 
 int defl_trace_TD_gamma(dtr_defl_s *D, unsigned want, cudaStream_t st) {

@@ -127,15 +127,19 @@ __global__ void __launch_bounds__(256)
     }
   }
 }
-// from the largest fields to exponents; least: smallest exponent whose integers keep every bit of the storage type
+// from the largest fields to exponents (one block); least: smallest exponent whose integers keep every bit of the storage
+// type; *bad: whether any column fails
 __global__ void k_oz_exp_finish(int *stat, int cols, int bias, int top, int least, int *bad) {
-  for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < cols; c += gridDim.x * blockDim.x) {
+  int any = 0;
+  for (int c = threadIdx.x; c < cols; c += blockDim.x) {
     const int s = stat[c];
     const int e = s == 0 ? kZero : s - 1 >= top ? kBad : s - 1 - bias + 1;
     const bool b = e == kBad || (e != kZero && e < least);
     stat[c] = b ? kBad : e == kZero ? 0 : e;
-    if (b) *bad = 1;
+    any |= b;
   }
+  any = __syncthreads_or(any);
+  if (threadIdx.x == 0) *bad = any ? 1 : 0;
 }
 
 // ------------------------------------------------------------------- mma
@@ -499,31 +503,24 @@ __global__ void __launch_bounds__(256, 2)
 }
 
 // --------------------------------------------------------------- launchers
-// per-vector exponents of a deflation space into D->vexp, D->vexp_ok if every column can be written in integers
-int defl_oz_setup(dtr_defl_s *D, cudaStream_t st) {
-  D->vexp_ok = false;
-  if (!D->vexp) return DTR_OK;
+// per-vector exponents of a deflation space into D->vexp
+int defl_oz_setup(const dtr_defl_s *D, int *bad, cudaStream_t st) {
   const int k = D->k;
   const int64_t N = D->lat.N;
-  int *bad = D->vexp + k;
-  DTR_CUDA(cudaMemsetAsync(D->vexp, 0, (k + 1) * sizeof(int), st));
+  DTR_CUDA(cudaMemsetAsync(D->vexp, 0, k * sizeof(int), st));
   const unsigned grid = (unsigned)(8 * device_sms());
   // (an FP32 entry is exact down to 2^-31 of its column's largest; with an exponent of at least -60 subnormals are below)
   if (D->prec == DTR_F64) {
     k_oz_exp<double2><<<grid, 256, 0, st>>>((const double2 *)D->V, N, k, D->vexp, nullptr);
-    k_oz_exp_finish<<<4, 256, 0, st>>>(D->vexp, k, 1023, 0x7ff, -800, bad);
+    k_oz_exp_finish<<<1, 256, 0, st>>>(D->vexp, k, 1023, 0x7ff, -800, bad);
   } else {
     if (D->prec == DTR_F32)
       k_oz_exp<float2><<<grid, 256, 0, st>>>((const float2 *)D->V, N, k, D->vexp, nullptr);
     else
       k_oz_exp<bfc2><<<grid, 256, 0, st>>>((const bfc2 *)D->V, N, k, D->vexp, nullptr);
-    k_oz_exp_finish<<<4, 256, 0, st>>>(D->vexp, k, 127, 0xff, -60, bad);
+    k_oz_exp_finish<<<1, 256, 0, st>>>(D->vexp, k, 127, 0xff, -60, bad);
   }
   count_launches(2);
-  int h = 1;
-  DTR_CUDA(cudaMemcpyAsync(&h, bad, sizeof(int), cudaMemcpyDeviceToHost, st));
-  DTR_CUDA(cudaStreamSynchronize(st));
-  D->vexp_ok = h == 0;
   return DTR_OK;
 }
 

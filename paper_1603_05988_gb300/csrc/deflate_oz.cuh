@@ -5,8 +5,9 @@
 
 namespace dtr {
 
-// Exponents of V's columns into D->vexp (k + 1 ints, device); D->vexp_ok: every column can be written in integers.
-int defl_oz_setup(dtr_defl_s *D, cudaStream_t st);
+// Queues the exponents of V's columns into D->vexp (k ints, device); *bad (device): some column cannot be written in
+// integers.
+int defl_oz_setup(const dtr_defl_s *D, int *bad, cudaStream_t st);
 size_t defl_oz_scratch_bytes(int k, int b);
 // Partial sums as k_defl_partial's, over *chunks (<= max_chunks) chunks of sites.
 int defl_oz_contract(const dtr_defl_s *D, const double2 *Z, int b, void *scratch, int max_chunks, double2 *partial,
