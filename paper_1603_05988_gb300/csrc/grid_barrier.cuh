@@ -7,8 +7,8 @@
 namespace dtr {
 
 constexpr long long kSpinBudget = 4000000000LL;  // ~2 s at 2 GHz
-// Largest persistent grid: two buffers of 5 x 64 partials per block fit the
-// solver's reduction scratch (kMaxGrid x 5 x 64 double2).
+// Largest persistent grid: two buffers of partials per block, 5 x 64 double2 (whole lattice) or 8 x 64 float or double
+// (red-black), fit the solver's reduction scratch (kMaxGrid x 5 x 64 double2).
 constexpr int kPersistMaxGrid = kMaxGrid / 2;
 
 __device__ __forceinline__ unsigned long long global_ns() {

@@ -222,7 +222,8 @@ __global__ void __launch_bounds__(kBlock) k_eo_split(const double2 *__restrict__
   }
 }
 
-// inner problem: r = rhat = p = fac (r_e + H r_o / (2 D)), e = 0 on the even sites; the inner scalars, with
+// inner problem: r = rhat = p = fac (r_e + H r_o / (2 D)), e = 0 on the even sites, from the hi parts of the residual alone
+// (truncated, not rounded, to 24 bits: the next outer residual takes that up with the rest); the inner scalars, with
 // rho = |r|^2 and the norm that the tolerance refers to that of the whole residual
 template <typename S>
 __global__ void __launch_bounds__(kBlock, 2) k_eo_init(const float2 *__restrict__ U, const float4 *__restrict__ res,
@@ -360,8 +361,9 @@ __global__ void __launch_bounds__(kBlock, 2) k_eo_accum(const float2 *__restrict
 // Residual after a cycle without a stencil on x: x grew by e / (base fac), so r -= A e / fac, A e in double-float
 // (links split into hi and lo, e exact in FP32): relative error ~2^-46 of |A| |e|, so r stays the true residual of x
 // to ~1e-14 kappa |z| over all cycles; a true residual confirms convergence before it is reported.
-// FP32 arithmetic and load latency bound it: two blocks to an SM (128 registers, ~150 B spilled) 8.9 ms against 9.8 ms for
-// one (232 registers) at 32^3 x 64 x 16; a loop over directions that needs no spills took 10.9 ms.
+// FP32 arithmetic and load latency bound it: two blocks to an SM (128 registers, ~150 B spilled) 13.4 ms against 14.7 ms
+// for one (232 registers) at 32^3 x 64 x 16, each of the two that run in a solve; a loop over directions that needs no
+// spills took 16.3 ms.
 __global__ void __launch_bounds__(kBlock, 2) k_eo_update(const float4 *__restrict__ Udf, const float4 *__restrict__ e,
                                                          float4 *__restrict__ rhi, float4 *__restrict__ rlo, Blk k,
                                                          float dhi, float dlo, Scal *sc, Reduce red, double hs,
@@ -402,7 +404,8 @@ __global__ void __launch_bounds__(kBlock, 2) k_eo_update(const float4 *__restric
 
 // True residual r = base (z - A x) with A x in double-float on the split x: each component carries an error of about
 // 2^-46 times the sum of the stencil terms' magnitudes (~9 |x|), i.e. ~1e-13 |x| / |z| relative to z, a hundredth of a
-// 1e-10 tolerance while |x| / |z| stays below ~10.  One block to an SM: 3.0 ms at 32^3 x 64 x 16, two 3.3 ms.
+// 1e-10 tolerance while |x| / |z| stays below ~10.  One block to an SM: 15.1 ms at 32^3 x 64 x 16 where it runs (once a
+// solve), two blocks 16.5 ms.
 __global__ void __launch_bounds__(kBlock, 1) k_eo_resid_df(const float4 *__restrict__ Udf,
                                                            const float4 *__restrict__ xhi,
                                                            const float4 *__restrict__ xlo,

@@ -7,7 +7,8 @@
 namespace dtr {
 
 // Device buffers of one block's cycles, all in the pair layout of eo_core.cuh over bi = max(b, 2) columns: "both" is
-// [parity][h][12][bi / 2] float4 (even sites first), "half" [h][12][bi / 2] in the storage of the Krylov vectors.
+// [parity][h][12][bi / 2] float4 (even sites first), "half" [h][12][bi / 2] in the storage of the Krylov vectors, but w,
+// on the odd sites, in FP32.
 struct EoBufs {
   float4 *rhi, *rlo;               // both: the residual times base, in double-float
   float4 *e;                       // both: the cycle's correction times base * fac
@@ -19,8 +20,9 @@ size_t eo_scratch_bytes(int64_t V, int b);
 // hands out the buffers in eo_scratch_bytes bytes from a 256-byte-aligned address
 EoBufs eo_carve(char *w, int64_t V, int b);
 
-// Schur complement usable: it divides by D = 4 + m0, and entries of w = H p / (2 D) stay within 8 of p's down to
-// |D| = 1/2.
+// Schur complement usable: it divides by D = 4 + m0, and ||w|| = ||H p|| / (2 |D|) stays within 8 ||p|| down to |D| = 1/2.
+// At |D| <= 2 BiCGStab converged on neither system (4^4 to 8^3 x 16, eps 0.2 and 0.7, every storage), so the line's
+// place there decides nothing but which kernels run out of iterations.
 inline bool eo_usable(double m0) { return (4.0 + m0) * (4.0 + m0) >= 0.25; }
 
 struct EoSolve {
