@@ -111,9 +111,12 @@ __device__ __forceinline__ bool is_zero(bfc2 v) { return is_zero(__bfloat1622flo
 template <typename T>
 __global__ void __launch_bounds__(256)
     k_oz_exp(const T *__restrict__ F, int64_t rows, int cols, int *__restrict__ stat, int *__restrict__ count) {
+  __shared__ int most[256], number[256];
   for (int c0 = 0; c0 < cols; c0 += 256) {
     const int w = min(256, cols - c0), g = 256 / w;  // g rows of w columns at once
     const int c = threadIdx.x % w, r = threadIdx.x / w;
+    most[threadIdx.x] = number[threadIdx.x] = 0;
+    __syncthreads();
     if (r < g) {
       int m = 0, n = 0;
       for (int64_t i = (int64_t)blockIdx.x * g + r; i < rows; i += (int64_t)gridDim.x * g) {
@@ -122,21 +125,32 @@ __global__ void __launch_bounds__(256)
         m = max(m, 1 + exp_field(v));
         ++n;
       }
-      if (m) atomicMax(&stat[c0 + c], m);  // (neither the largest nor the count depends on the order)
-      if (n && count) atomicAdd(&count[c0 + c], n);
+      if (m) atomicMax(&most[c], m);  // (neither the largest nor the count depends on the order)
+      if (n) atomicAdd(&number[c], n);
     }
+    __syncthreads();
+    if (threadIdx.x < w && number[threadIdx.x]) {
+      atomicMax(&stat[c0 + threadIdx.x], most[threadIdx.x]);
+      if (count) atomicAdd(&count[c0 + threadIdx.x], number[threadIdx.x]);
+    }
+    __syncthreads();
   }
 }
-// from the largest fields to exponents (one block); least: smallest exponent whose integers keep every bit of the storage
-// type; *bad: whether any column fails
+// From a largest field (stat) to the exponent, 0 for a zero column, kBad; least: smallest exponent whose integers keep
+// every bit of the storage type.
+__device__ __forceinline__ int exp_of(int s, int bias, int top, int least) {
+  if (s == 0) return 0;
+  const int e = s - 1 - bias + 1;
+  return s - 1 >= top || e < least ? kBad : e;
+}
+__device__ __forceinline__ int exp_of_z(int s) { return exp_of(s, 1023, 0x7ff, -800); }
+// all columns' (one block); *bad: whether any column fails
 __global__ void k_oz_exp_finish(int *stat, int cols, int bias, int top, int least, int *bad) {
   int any = 0;
   for (int c = threadIdx.x; c < cols; c += blockDim.x) {
-    const int s = stat[c];
-    const int e = s == 0 ? kZero : s - 1 >= top ? kBad : s - 1 - bias + 1;
-    const bool b = e == kBad || (e != kZero && e < least);
-    stat[c] = b ? kBad : e == kZero ? 0 : e;
-    any |= b;
+    const int e = exp_of(stat[c], bias, top, least);
+    stat[c] = e;
+    any |= e == kBad;
   }
   any = __syncthreads_or(any);
   if (threadIdx.x == 0) *bad = any ? 1 : 0;
@@ -239,20 +253,21 @@ __device__ __forceinline__ unsigned mag(double2 v, int e) {
 __device__ __forceinline__ unsigned mag(bfc2 v, int e) { return mag(__bfloat1622float2(v), e); }
 
 // mass[m b + j] += 2^16 sum over sites of |v| |z| (moduli as above: a lower bound, so part of the sites may do); the last
-// block compares with sqrt(n / 2) and sets *fail for a pair that falls short.  Sites: every step-th (REST = false), or all
-// but these (run if *need is set).  A block: 64 vectors x 16 columns, stages of 4 sites as BF16 in shared memory; eight
-// warps of 16 x 8 sums.
+// block compares with sqrt(n / 2) and sets *fail for a pair that falls short.  Sites: every step-th (REST = false: here z
+// still holds k_oz_exp's fields, which the last block turns into exponents, setting *bad), or all but these (run if *need
+// is set).  A block: 64 vectors x 16 columns, stages of 4 sites as BF16 in shared memory; eight warps of 16 x 8 sums.  Its
+// loads are issued together, past the ends too (on valid entries, not used): one by one behind their tests a stage took
+// 8 us instead of 2.
 constexpr int kMM = 64, kMJ = 16, kMK = 48;
 constexpr int kMAs = (kMM + 8) * 2, kMBs = (kMJ + 8) * 2;  // bytes of a dof row
 template <typename VC, bool REST>
 __global__ void __launch_bounds__(256)
     k_oz_mass(const VC *__restrict__ Vd, const int *__restrict__ ev, const double2 *__restrict__ Z,
-              const int *__restrict__ ez, const int *__restrict__ count, const int *__restrict__ bad,
-              const int *__restrict__ need, int k, int b, int nsites, int step, unsigned long long *__restrict__ mass,
-              unsigned *__restrict__ arrived, int *fail) {
+              int *ez, const int *__restrict__ count, int *bad, const int *__restrict__ need, int k, int b, int nsites,
+              int step, unsigned long long *__restrict__ mass, unsigned *__restrict__ arrived, int *fail) {
   __shared__ __align__(16) unsigned char sm[kMK * (kMAs + kMBs)];
   __shared__ int last;
-  if (*bad || (REST && !*need)) return;  // (settled by the kernels before: the same for all blocks)
+  if (REST && (*bad || !*need)) return;  // (settled by the kernel before: the same for all blocks)
   unsigned short *As = (unsigned short *)sm, *Bs = (unsigned short *)(sm + kMK * kMAs);
   const int first = (nsites + step - 1) / step, total = REST ? nsites - first : first;
   const int i0 = (int)((int64_t)total * blockIdx.x / gridDim.x), i1 = (int)((int64_t)total * (blockIdx.x + 1) / gridDim.x);
@@ -260,30 +275,38 @@ __global__ void __launch_bounds__(256)
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int am = threadIdx.x % kMM, ad = threadIdx.x / kMM, bj = threadIdx.x % kMJ, bd = threadIdx.x / kMJ;
   const bool va = m0 + am < k, vb = j0 + bj < b;
-  const int ea = va ? ev[m0 + am] : 0, eb = vb ? ez[j0 + bj] : 0;
+  const int ma = va ? m0 + am : k - 1, jb = vb ? j0 + bj : b - 1;
+  const int ea = ev[ma], eb = REST ? ez[jb] : exp_of_z(ez[jb]);
   const unsigned base = (unsigned)__cvta_generic_to_shared(sm);
   const unsigned a_addr = base + ((lane >> 4) * 8 + (lane & 7)) * kMAs + ((w & 3) * 16 + (lane >> 3 & 1) * 8) * 2;
   const unsigned b_addr = base + kMK * kMAs + (lane & 15) * kMBs + (w >> 2) * 16;
   float c[4] = {0.f, 0.f, 0.f, 0.f};
   for (int i = i0; i < i1; i += 4) {
-    unsigned a[kMK * kMM / 256], z[kMK * kMJ / 256];
+    VC a[kMK * kMM / 256];
+    double2 z[kMK * kMJ / 256];
 #pragma unroll
     for (int u = 0; u < kMK * kMM / 256; ++u) {
-      const int d = ad + u * (256 / kMM), q = i + d / 12;
+      const int d = ad + u * (256 / kMM), q = min(i + d / 12, i1 - 1);
       const int64_t s = REST ? q + q / (step - 1) + 1 : (int64_t)q * step;
-      a[u] = q < i1 && va ? mag(Vd[(s * 12 + d % 12) * k + m0 + am], ea) : 0u;
+      a[u] = Vd[(s * 12 + d % 12) * k + ma];
     }
 #pragma unroll
     for (int u = 0; u < kMK * kMJ / 256; ++u) {
-      const int d = bd + u * (256 / kMJ), q = i + d / 12;
+      const int d = bd + u * (256 / kMJ), q = min(i + d / 12, i1 - 1);
       const int64_t s = REST ? q + q / (step - 1) + 1 : (int64_t)q * step;
-      z[u] = q < i1 && vb ? mag(Z[(s * 12 + d % 12) * b + j0 + bj], eb) : 0u;
+      z[u] = Z[(s * 12 + d % 12) * b + jb];
     }
     __syncthreads();
 #pragma unroll
-    for (int u = 0; u < kMK * kMM / 256; ++u) As[(ad + u * (256 / kMM)) * (kMAs / 2) + am] = (unsigned short)a[u];
+    for (int u = 0; u < kMK * kMM / 256; ++u) {
+      const int d = ad + u * (256 / kMM);
+      As[d * (kMAs / 2) + am] = (unsigned short)(va && i + d / 12 < i1 ? mag(a[u], ea) : 0u);
+    }
 #pragma unroll
-    for (int u = 0; u < kMK * kMJ / 256; ++u) Bs[(bd + u * (256 / kMJ)) * (kMBs / 2) + bj] = (unsigned short)z[u];
+    for (int u = 0; u < kMK * kMJ / 256; ++u) {
+      const int d = bd + u * (256 / kMJ);
+      Bs[d * (kMBs / 2) + bj] = (unsigned short)(vb && i + d / 12 < i1 ? mag(z[u], eb) : 0u);
+    }
     __syncthreads();
 #pragma unroll
     for (int q = 0; q < kMK / 16; ++q) {
@@ -310,6 +333,11 @@ __global__ void __launch_bounds__(256)
   for (int e = threadIdx.x; e < k * b; e += 256)
     low |= (float)__ldcg(&mass[e]) < 65536.f * sqrtf(0.5f * (float)count[e % b]);
   if (__syncthreads_or(low) && threadIdx.x == 0) *fail = 1;
+  if (!REST && threadIdx.x < b) {
+    const int e = exp_of_z(ez[threadIdx.x]);
+    ez[threadIdx.x] = e;
+    if (e == kBad) *bad = 1;
+  }
 }
 
 // ------------------------------------------------------------ contraction
@@ -550,7 +578,7 @@ template <typename VC> static int mass_t(const dtr_defl_s *D, const double2 *Z, 
   const int tiles = ((k + kMM - 1) / kMM) * ((b + kMJ - 1) / kMJ);
   auto grid = [&](int sites) {
     int n = (4 * device_sms() + tiles - 1) / tiles;
-    if (n > (sites + 15) / 16) n = (sites + 15) / 16;
+    if (n > (sites + 3) / 4) n = (sites + 3) / 4;
     return dim3(n < 1 ? 1 : n, (k + kMM - 1) / kMM, (b + kMJ - 1) / kMJ);
   };
   unsigned long long *mass = (unsigned long long *)(sc + kMass);
@@ -586,8 +614,7 @@ int defl_oz_contract(const dtr_defl_s *D, const double2 *Z, int b, void *scratch
   const int V = (int)D->lat.V, sms = device_sms();
   DTR_CUDA(cudaMemsetAsync(sc, 0, planes_at(D->k, b) * sizeof(int), st));
   k_oz_exp<double2><<<(unsigned)(8 * sms), 256, 0, st>>>(Z, (int64_t)V * 12, b, sc + kEz, sc + kCount);
-  k_oz_exp_finish<<<1, 64, 0, st>>>(sc + kEz, b, 1023, 0x7ff, -800, sc + kBadC);
-  count_launches(2);
+  count_launches(1);
   const int tiles = 2 * ((D->k + kOM - 1) / kOM) * ((b + kOJ - 1) / kOJ);
   int nch = (4 * sms + tiles - 1) / tiles;  // about two rounds of two blocks to an SM
   if (nch > V / 16) nch = V / 16 > 0 ? V / 16 : 1;
