@@ -365,7 +365,8 @@ int dtr_defl_to_host(dtr_defl d, double *V_host, double *lambda_host);
  * coeff_out: device k x 2 nrhs complex128 column-major, or NULL.
  * x0_out: device canonical N x nrhs, or NULL: receives the deflated solution
  *   V diag(1/lambda) V^H gamma_5 z = A_D^-1 z.
- * Accuracy: that of FP64 sums, C to about 2^-53 of sum |v| |z|.  Larger blocks run on the tensor cores in integers
+ * Accuracy: that of FP64 sums, C to about 2^-53 of sum |v| |z|, x0 to about 2^-50 of the norm of every 16 neighbouring
+ * entries.  Larger blocks run on the tensor cores in integers
  * relative to each column's largest entry, with 54 bits; blocks for which that would lose digits (entries small in V
  * where z is large or the other way round, point sources, solutions x0 that are small over a whole neighbourhood of 16
  * dofs; not finite values) are found on the device and take FP64 sums, at the FP64 pipe's rate.  So does a workspace

@@ -12,6 +12,7 @@
 #include <vector>
 
 #include "deflate.cuh"
+#include "deflate_oz.cuh"
 #include "dtr_internal.cuh"
 #include "net.cuh"
 #include "persist.cuh"
@@ -505,7 +506,7 @@ int dtr_defl_create(dtr_lattice lat, int k, dtr_prec prec, const double *V_host,
   D->inv_lambda = nullptr;
   std::vector<double> inv(k);
   for (int m = 0; m < k; ++m) inv[m] = 1.0 / lambda_host[m];
-  cudaError_t e = cudaMalloc(&D->inv_lambda, k * sizeof(double) + k * sizeof(int));
+  cudaError_t e = cudaMalloc(&D->inv_lambda, k * sizeof(double) + defl_oz_space_bytes(k));
   D->vexp = (int *)(D->inv_lambda + k);
   D->vexp_ok = false;
   if (e == cudaSuccess) e = cudaMemcpy(D->inv_lambda, inv.data(), k * sizeof(double), cudaMemcpyHostToDevice);
@@ -592,7 +593,7 @@ int dtr_eig_deflation(dtr_gauge g, double m0, const dtr_eig_params *p, void *wor
   D->inv_lambda = nullptr;
   // the basis of nb columns lives in the handle's buffer and is compacted to k columns at the end
   cudaError_t e = cudaMalloc(&D->V, (size_t)g->lat.N * nb * es);
-  if (e == cudaSuccess) e = cudaMalloc(&D->inv_lambda, p->k * sizeof(double) + p->k * sizeof(int));
+  if (e == cudaSuccess) e = cudaMalloc(&D->inv_lambda, p->k * sizeof(double) + defl_oz_space_bytes(p->k));
   D->vexp = (int *)(D->inv_lambda + p->k);
   D->vexp_ok = false;
   if (e != cudaSuccess) {

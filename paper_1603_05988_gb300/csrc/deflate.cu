@@ -439,8 +439,9 @@ int defl_trace_TD(dtr_defl_s *D, cudaStream_t st) {
   const int nch = (int)nch64;
   double *part = nullptr, *td = nullptr;
   D->vexp_ok = false;
-  DTR_CUDA(cudaMalloc((void **)&part, (size_t)nch * k * sizeof(double) + 256));
-  td = (double *)((char *)part + (((size_t)nch * k * sizeof(double) + 127) / 128) * 128);
+  const size_t psize = (size_t)(nch > 2 ? nch : 2) * k * sizeof(double);  // (at least the digits' 12 k bytes)
+  DTR_CUDA(cudaMalloc((void **)&part, psize + 256));
+  td = (double *)((char *)part + (psize + 127) / 128 * 128);
   const dim3 grid(nch, mt);
   if (D->prec == DTR_F64)
     k_defl_td_partial<double2><<<grid, kTdThreads, 0, st>>>((const double2 *)D->V, k, nsite, nch, part);
@@ -450,13 +451,13 @@ int defl_trace_TD(dtr_defl_s *D, cudaStream_t st) {
     k_defl_td_partial<bfc2><<<grid, kTdThreads, 0, st>>>((const bfc2 *)D->V, k, nsite, nch, part);
   count_launches(1);
   k_defl_td_reduce<<<1, kTdThreads, 0, st>>>(part, D->inv_lambda, k, nch, td); count_launches(1);
-  // the digits' exponents, waited for together with T_D
-  const int rc = defl_oz_setup(D, (int *)(td + 1), st);
+  // what the digits need, waited for together with T_D
+  const int rc = defl_oz_setup(D, part, (int *)(td + 1), st);
   cudaError_t e = cudaGetLastError();
   struct {
     double td;
-    int bad, pad;
-  } h = {0.0, 1, 0};
+    int bad, lossy;
+  } h = {0.0, 1, 1};
   if (e == cudaSuccess) e = cudaMemcpyAsync(&h, td, sizeof(h), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   cudaFree(part);
@@ -465,6 +466,7 @@ int defl_trace_TD(dtr_defl_s *D, cudaStream_t st) {
   D->td[0] = h.td;
   D->td[1] = 0.0;
   D->vexp_ok = h.bad == 0;
+  D->vlossy = h.lossy != 0;
   return DTR_OK;
 }
 

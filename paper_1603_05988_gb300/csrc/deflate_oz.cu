@@ -13,13 +13,16 @@
 // Integers are fixed point where FP64 floats: an entry is off by up to 2^-55 of its column's largest, so a product of two
 // entries that are both small for their columns loses digits.  Two tests on the device send such blocks to the FP64
 // kernels (a point source; vectors that decay from opposite ends):
-//   C   S = sum of the products of the entries' moduli, in units of the columns' powers of two, must reach
-//       sqrt(n / 2) for n nonzero entries of z (k_oz_mass).  The digits' error is then below 0.06 2^-53 of
-//       sum |v| |z|; FP64 chains come to 0.02 to 0.2 (49152 dofs, 18 families of graded, localised, sparse and plain
-//       columns).  Gaussian columns reach 4.4 sqrt(n) there, growing with sqrt(n).
-//   x0  sixteen neighbouring entries of a column must have an RMS of 2^-7.5 sqrt(k) in the weights' units, 2^-6.5 if V is
-//       FP64 (k_oz_expand).  Their error is then below 2^-50 of their norm (largest seen 6e-16; FP64 sums 1e-15 at
-//       k = 200).  Gaussian V and weights over three decades reach 2^-6.2 and more.
+//   C   S = sum of the products of the entries' moduli, in units of the columns' powers of two, must reach a bound T
+//       (k_oz_mass).  The digits' error goes with the squares that meet a rounded partner: T^2 = 4 (sum |v|^2 + sum |z|^2 where
+//       v is rounded + 2^-13 n for the dropped pairs), or n / 2 for n nonzero entries of z if that is less.  At S = T it is
+//       0.06 2^-53 of sum |v| |z|; FP64 chains come to 0.02 to 0.3 (49152 dofs, 24 families of graded, localised, sparse
+//       and plain columns).  Gaussian columns reach 6 T (FP64) and 12 T (FP32) there, growing with sqrt(n).
+//   x0  sixteen neighbouring entries of a column, together, must be 2^50 times the error that they can have: that of V's
+//       entries where V is FP64 (2^-55 / sqrt(3) of the columns' powers of two, times the weights), and the digit pairs that
+//       are dropped (k_oz_expand).  FP32 and BF16 entries are exact in 54 bits down to 2^-30 of the largest, so that only the
+//       latter counts.  Largest errors of 16 entries above the line 7e-16, FP64 sums 9e-16 (spaces of the eigensolver, 8^4 to
+//       16^3 x 32, k = 16 to 100); its spaces at 16^4, FP64, are partly below.
 //
 // Digits come from shifts and byte permutes on the integer pipe.  A digit plane of Z that is zero over a stage is
 // skipped: probing noise (entries 0, +-1, +-i) has one digit.
@@ -69,6 +72,21 @@ __device__ __forceinline__ Dig2 dig(float2 v, int e) { return Dig2{digits_of(v.x
 __device__ __forceinline__ Dig2 dig(double2 v, int e) { return Dig2{digits_of(v.x, e), digits_of(v.y, e)}; }
 __device__ __forceinline__ Dig2 dig(bfc2 v, int e) { return dig(__bfloat1622float2(v), e); }
 constexpr unsigned long long kNoDig = 0x0080808080808080ull;
+// entry times 2^-e
+__device__ __forceinline__ float2 scaled(float2 v, int e) { return make_float2(ldexpf(v.x, -e), ldexpf(v.y, -e)); }
+__device__ __forceinline__ float2 scaled(double2 v, int e) {
+  return f64_to_f32(make_double2(scalbn(v.x, -e), scalbn(v.y, -e)));
+}
+__device__ __forceinline__ float2 scaled(bfc2 v, int e) { return scaled(__bfloat1622float2(v), e); }
+// whether the integer of an FP32 (or BF16) entry loses bits
+__device__ __forceinline__ int loses_bits(float f, int e) {
+  const unsigned b = __float_as_uint(f) & 0x7fffffffu;
+  const int x = (int)(b >> 23), sh = x - 150 + kIntBits - e;
+  return sh < 0 && b != 0u && (x == 0 || sh <= -24 || (b & ((1u << -sh) - 1u)) != 0u);
+}
+__device__ __forceinline__ int loses_bits(float2 v, int e) { return loses_bits(v.x, e) + loses_bits(v.y, e); }
+__device__ __forceinline__ int loses_bits(bfc2 v, int e) { return loses_bits(__bfloat1622float2(v), e); }
+__device__ __forceinline__ int loses_bits(double2, int) { return 0; }  // (nearly all do: not counted)
 
 // digit i of a biased integer as a float (exact): 2^23 + byte, minus 2^23 + 128
 __device__ __forceinline__ float digit(unsigned long long q, int i) {
@@ -144,7 +162,7 @@ __device__ __forceinline__ int exp_of(int s, int bias, int top, int least) {
   return s - 1 >= top || e < least ? kBad : e;
 }
 __device__ __forceinline__ int exp_of_z(int s) { return exp_of(s, 1023, 0x7ff, -800); }
-// all columns' (one block); *bad: whether any column fails
+// all columns' (one block); bad[0]: whether any column fails, bad[1]: 0
 __global__ void k_oz_exp_finish(int *stat, int cols, int bias, int top, int least, int *bad) {
   int any = 0;
   for (int c = threadIdx.x; c < cols; c += blockDim.x) {
@@ -153,7 +171,52 @@ __global__ void k_oz_exp_finish(int *stat, int cols, int bias, int top, int leas
     any |= e == kBad;
   }
   any = __syncthreads_or(any);
-  if (threadIdx.x == 0) *bad = any ? 1 : 0;
+  if (threadIdx.x == 0) bad[0] = any ? 1 : 0, bad[1] = 0;
+}
+
+// sq[m] += 2^32 sum |v|^2 of column m in units of its power of two, lost[m]: entries that lose bits
+template <typename T>
+__global__ void __launch_bounds__(256)
+    k_oz_squares(const T *__restrict__ F, int64_t rows, int cols, const int *__restrict__ ev,
+                 unsigned long long *__restrict__ sq, int *__restrict__ lost) {
+  __shared__ unsigned long long sum[256];
+  __shared__ int number[256];
+  for (int c0 = 0; c0 < cols; c0 += 256) {
+    const int w = min(256, cols - c0), g = 256 / w;
+    const int c = threadIdx.x % w, r = threadIdx.x / w;
+    sum[threadIdx.x] = 0;
+    number[threadIdx.x] = 0;
+    __syncthreads();
+    if (r < g) {
+      const int e = ev[c0 + c];
+      float s = 0.f;
+      int n = 0;
+      for (int64_t i = (int64_t)blockIdx.x * g + r; i < rows; i += (int64_t)gridDim.x * g) {
+        const T v = F[i * cols + c0 + c];
+        const float2 u = scaled(v, e);
+        s = fmaf(u.x, u.x, fmaf(u.y, u.y, s));
+        n += loses_bits(v, e);
+      }
+      atomicAdd(&sum[c], (unsigned long long)(s * 4294967296.f));
+      if (n) atomicAdd(&number[c], n);
+    }
+    __syncthreads();
+    if (threadIdx.x < w) {
+      atomicAdd(&sq[c0 + threadIdx.x], sum[threadIdx.x]);
+      if (number[threadIdx.x]) atomicAdd(&lost[c0 + threadIdx.x], number[threadIdx.x]);
+    }
+    __syncthreads();
+  }
+}
+// v2[m]: the sum, lost2[m]: largest sum of squares that can meet a rounded entry of v (FP64 spaces: no limit); *lossy: set
+// if a column has entries that lose bits
+__global__ void k_oz_limits(const unsigned long long *__restrict__ sq, const int *__restrict__ lost, int cols, bool rounded,
+                            float *__restrict__ v2, float *__restrict__ lost2, int *lossy) {
+  for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < cols; c += gridDim.x * blockDim.x) {
+    v2[c] = (float)sq[c] * 0x1p-32f;
+    lost2[c] = rounded ? 3e38f : 2.f * (float)lost[c];
+    if (lost[c]) *lossy = 1;
+  }
 }
 
 // ------------------------------------------------------------------- mma
@@ -252,8 +315,8 @@ __device__ __forceinline__ unsigned mag(double2 v, int e) {
 }
 __device__ __forceinline__ unsigned mag(bfc2 v, int e) { return mag(__bfloat1622float2(v), e); }
 
-// mass[m b + j] += 2^16 sum over sites of |v| |z| (moduli as above: a lower bound, so part of the sites may do); the last
-// block compares with sqrt(n / 2) and sets *fail for a pair that falls short.  Sites: every step-th (REST = false: here z
+// mass[m b + j] += 2^16 sum over sites of |v| |z| (moduli as above: a lower bound, so part of the sites may do), z2[j] +=
+// sum |z|^2 (an upper bound); the last block compares with T and sets *fail for a pair that falls short.  Sites: every step-th (REST = false: here z
 // still holds k_oz_exp's fields, which the last block turns into exponents, setting *bad), or all but these (run if *need
 // is set).  A block: 64 vectors x 16 columns, stages of 4 sites as BF16 in shared memory; eight warps of 16 x 8 sums.  Its
 // loads are issued together, past the ends too (on valid entries, not used): one by one behind their tests a stage took
@@ -264,8 +327,10 @@ template <typename VC, bool REST>
 __global__ void __launch_bounds__(256)
     k_oz_mass(const VC *__restrict__ Vd, const int *__restrict__ ev, const double2 *__restrict__ Z,
               int *ez, const int *__restrict__ count, int *bad, const int *__restrict__ need, int k, int b, int nsites,
-              int step, unsigned long long *__restrict__ mass, unsigned *__restrict__ arrived, int *fail) {
+              int step, const float *__restrict__ v2, const float *__restrict__ lost2,
+              unsigned long long *__restrict__ mass, unsigned *__restrict__ z2, unsigned *__restrict__ arrived, int *fail) {
   __shared__ __align__(16) unsigned char sm[kMK * (kMAs + kMBs)];
+  __shared__ float zsum[8][kMJ];
   __shared__ int last;
   if (REST && (*bad || !*need)) return;  // (settled by the kernel before: the same for all blocks)
   unsigned short *As = (unsigned short *)sm, *Bs = (unsigned short *)(sm + kMK * kMAs);
@@ -280,7 +345,7 @@ __global__ void __launch_bounds__(256)
   const unsigned base = (unsigned)__cvta_generic_to_shared(sm);
   const unsigned a_addr = base + ((lane >> 4) * 8 + (lane & 7)) * kMAs + ((w & 3) * 16 + (lane >> 3 & 1) * 8) * 2;
   const unsigned b_addr = base + kMK * kMAs + (lane & 15) * kMBs + (w >> 2) * 16;
-  float c[4] = {0.f, 0.f, 0.f, 0.f};
+  float c[4] = {0.f, 0.f, 0.f, 0.f}, zz = 0.f;
   for (int i = i0; i < i1; i += 4) {
     VC a[kMK * kMM / 256];
     double2 z[kMK * kMJ / 256];
@@ -305,7 +370,9 @@ __global__ void __launch_bounds__(256)
 #pragma unroll
     for (int u = 0; u < kMK * kMJ / 256; ++u) {
       const int d = bd + u * (256 / kMJ);
-      Bs[d * (kMBs / 2) + bj] = (unsigned short)(vb && i + d / 12 < i1 ? mag(z[u], eb) : 0u);
+      const unsigned q = vb && i + d / 12 < i1 ? mag(z[u], eb) : 0u;
+      Bs[d * (kMBs / 2) + bj] = (unsigned short)q;
+      zz = fmaf(__uint_as_float(q << 16), __uint_as_float(q << 16), zz);
     }
     __syncthreads();
 #pragma unroll
@@ -322,6 +389,14 @@ __global__ void __launch_bounds__(256)
     const int m = m0 + (w & 3) * 16 + (q >> 1) * 8 + (lane >> 2), j = j0 + (w >> 2) * 8 + (lane & 3) * 2 + (q & 1);
     if (m < k && j < b && c[q] > 0.f) atomicAdd(&mass[(int64_t)m * b + j], (unsigned long long)(c[q] * 65536.f));
   }
+  zz += __shfl_xor_sync(0xffffffffu, zz, 16);
+  if (lane < 16) zsum[w][lane] = zz;
+  __syncthreads();
+  if (blockIdx.y == 0 && threadIdx.x < kMJ && j0 + threadIdx.x < b) {
+    float s = 0.f;
+    for (int q = 0; q < 8; ++q) s += zsum[q][threadIdx.x];
+    atomicAdd(&z2[j0 + threadIdx.x], (unsigned)ceilf(2.04f * s));  // |z|^2 is at most twice the larger part's, cut by 2^-7
+  }
   __threadfence();
   __syncthreads();
   if (threadIdx.x == 0) last = atomicAdd(arrived, 1u) == gridDim.x * gridDim.y * gridDim.z - 1;
@@ -330,8 +405,12 @@ __global__ void __launch_bounds__(256)
   __threadfence();
   int low = 0;
 #pragma unroll 4
-  for (int e = threadIdx.x; e < k * b; e += 256)
-    low |= (float)__ldcg(&mass[e]) < 65536.f * sqrtf(0.5f * (float)count[e % b]);
+  for (int e = threadIdx.x; e < k * b; e += 256) {
+    const int j = e % b, m = e / b;
+    const float n = (float)count[j], met = REST || step == 1 ? (float)__ldcg(&z2[j]) : 2.f * n;
+    const float t2 = fminf(0.5f * n, 4.f * (v2[m] + fminf(met, lost2[m]) + 0x1p-13f * n));
+    low |= (float)__ldcg(&mass[e]) < 65536.f * sqrtf(t2);
+  }
   if (__syncthreads_or(low) && threadIdx.x == 0) *fail = 1;
   if (!REST && threadIdx.x < b) {
     const int e = exp_of_z(ez[threadIdx.x]);
@@ -424,10 +503,14 @@ __global__ void __launch_bounds__(256, 2)
 // -------------------------------------------------------------- expansion
 // Digit planes of the weights for x0 = V W: Wd[i][2 m + c][2 j + d] as BF16, from W[m][j] 2^ev[m], with rows (Re, Im) of
 // V's entry against columns (Re, Im) of x0: (Wr, Wi; -Wi, Wr); ew[j]: exponent of column j, kZero if it is zero; one
-// block a column.
+// block a column.  least[j]: smallest sum of squares of 16 entries (in the weights' units) for the digits to do, 16 times
+// 2^100 the mean square error of an entry: 2/3 2^-110 of the sum of the weights' squares where V is rounded, and, as
+// 2^-123 k, the dropped pairs (2^-62 sqrt(2 k)).
 __global__ void __launch_bounds__(256) k_oz_weights(const double2 *__restrict__ W, const int *__restrict__ ev, int k,
-                                                    int b, unsigned *__restrict__ Wd, int *__restrict__ ew, int *bad) {
+                                                    int b, bool rounded, unsigned *__restrict__ Wd, int *__restrict__ ew,
+                                                    float *__restrict__ least, int *bad) {
   __shared__ int emax, nz;
+  __shared__ float sh[256];
   const int j = blockIdx.x;
   if (threadIdx.x == 0) emax = -(1 << 20), nz = 0;
   __syncthreads();
@@ -445,8 +528,11 @@ __global__ void __launch_bounds__(256) k_oz_weights(const double2 *__restrict__ 
     if (e > 800 || e < -800) *bad = 1;  // not finite, or out of the integers' reach
   }
   const int64_t plane = (int64_t)2 * k * b;  // 32-bit pairs of a digit plane
+  float w2 = 0.f;
   for (int m = threadIdx.x; m < k; m += 256) {
     const double2 v = W[(int64_t)j * k + m];
+    const float re = f64_to_f32(scalbn(v.x, ev[m] - e)), im = f64_to_f32(scalbn(v.y, ev[m] - e));
+    w2 = fmaf(re, re, fmaf(im, im, w2));
     const Dig2 d = dig(v, e - ev[m]), n = dig(make_double2(-v.y, v.x), e - ev[m]);
 #pragma unroll
     for (int i = 0; i < kDig; ++i) {
@@ -454,21 +540,32 @@ __global__ void __launch_bounds__(256) k_oz_weights(const double2 *__restrict__ 
       Wd[i * plane + (int64_t)(2 * m + 1) * b + j] = digit_pair(n, i);
     }
   }
+  sh[threadIdx.x] = w2;
+  __syncthreads();
+  for (int o = 128; o > 0; o >>= 1) {
+    if ((int)threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) least[j] = 16.f * ((rounded ? (2.f / 3.f) * 0x1p-10f * sh[0] : 0.f) + 0x1p-23f * (float)k);
 }
 
 // x[dof][j] = sum_m V[dof][m] W[m][j]: a block takes 64 dofs x 16 columns, 32 vectors (64 rows of Wd) a stage.
-// *small is set where 16 dofs of a column have squares below `least` in sum (in the weights' units).
+// *small is set where 16 dofs of a column have squares below the column's `least` in sum (in the weights' units), with an
+// allowance for the FP32 and BF16 entries of the tile that lose bits (2/3 2^-110 each, for weights of at most one unit).
+// LOSSY: the space has such entries; looked for in any case, they cost 2 % of a projection.
 constexpr int kXD = 64, kXM = 32;
 constexpr int kXAs = (2 * kXM + 8) * 2, kXBs = (2 * kOJ + 8) * 2;
 constexpr int kXAp = kXD * kXAs, kXBp = 2 * kXM * kXBs;
 constexpr int kXBytes = kDig * (kXAp + kXBp);
-template <typename VC>
+template <typename VC, bool LOSSY>
 __global__ void __launch_bounds__(256, 2)
     k_oz_expand(const VC *__restrict__ Vd, const int *__restrict__ ev, const unsigned *__restrict__ Wd,
-                const int *__restrict__ ew, const int *__restrict__ bad, int k, int b, int64_t N, float least, int *small,
-                double2 *__restrict__ x) {
+                const int *__restrict__ ew, const int *__restrict__ bad, int k, int b, int64_t N,
+                const float *__restrict__ least, int *small, double2 *__restrict__ x) {
   extern __shared__ __align__(16) unsigned char sm[];
-  if (*bad) return;  // the FP64 kernel runs instead
+  __shared__ int lost[2];  // entries that lose bits, of this tile and (cleared) the next
+  if (*bad) return;        // the FP64 kernel runs instead
+  if (LOSSY && threadIdx.x < 2) lost[threadIdx.x] = 0;
   unsigned *As = (unsigned *)sm, *Bs = (unsigned *)(sm + kDig * kXAp);
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int j0 = blockIdx.y * kOJ;
@@ -481,20 +578,28 @@ __global__ void __launch_bounds__(256, 2)
   const int64_t plane = (int64_t)2 * k * b;
   const int64_t tiles = (N + kXD - 1) / kXD;
   const bool one = k <= kXM;  // the weights of all vectors stay in shared memory
-  for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+  int turn = 0;
+  for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x, turn ^= 1) {
     const int64_t i0 = tile * kXD;
     Acc acc;
     int stage = 0;
     for (int m0 = 0; m0 < k; m0 += kXM, ++stage) {
       __syncthreads();
+      if (LOSSY && m0 == 0 && threadIdx.x == 0) lost[turn ^ 1] = 0;
+      int mine = 0;
 #pragma unroll
       for (int u = 0; u < kXD * kXM / 256; ++u) {
         const int d = ad + u * (256 / kXM);
         Dig2 g{kNoDig, kNoDig};
-        if (i0 + d < N && m0 + am < k) g = dig(Vd[(i0 + d) * k + m0 + am], ev[m0 + am]);
+        if (i0 + d < N && m0 + am < k) {
+          const VC v = Vd[(i0 + d) * k + m0 + am];
+          g = dig(v, ev[m0 + am]);
+          if (LOSSY) mine += loses_bits(v, ev[m0 + am]);
+        }
 #pragma unroll
         for (int i = 0; i < kDig; ++i) As[(i * kXAp + d * kXAs) / 4 + am] = digit_pair(g, i);
       }
+      if (LOSSY && mine) atomicAdd(&lost[turn], mine);
       if (!one || tile == blockIdx.x) {
         for (int q = threadIdx.x; q < kDig * 2 * kXM * kOJ; q += 256) {
           const int j = q % kOJ, r = q / kOJ % (2 * kXM), i = q / (kOJ * 2 * kXM);
@@ -509,6 +614,7 @@ __global__ void __launch_bounds__(256, 2)
       if (stage & 1) acc.flush();  // 128 terms
     }
     acc.flush();
+    const float allow = LOSSY ? (2.f / 3.f) * 0x1p-10f * 16.f / kXD * (float)lost[turn] : 0.f;
 #pragma unroll
     for (int t = 0; t < 2; ++t) {
       const int j = j0 + ((w >> 2) * 16 + t * 8 + (lane & 3) * 2) / 2;
@@ -525,38 +631,51 @@ __global__ void __launch_bounds__(256, 2)
 #pragma unroll
       for (int o = 4; o < 32; o <<= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
       // (a warp's 16 dofs are all below N or none: N is a multiple of 192)
-      if (sq < least && e != kZero && i0 + (w & 3) * 16 < N) *small = 1;
+      if (e != kZero && i0 + (w & 3) * 16 < N && sq < least[j] + allow) *small = 1;
     }
   }
 }
 
 // --------------------------------------------------------------- launchers
-// per-vector exponents of a deflation space into D->vexp
-int defl_oz_setup(const dtr_defl_s *D, int *bad, cudaStream_t st) {
+// per-vector exponents of a deflation space into D->vexp, and what the mass test needs of it behind them
+size_t defl_oz_space_bytes(int k) { return 3 * (size_t)k * sizeof(int); }
+static float *space_v2(const dtr_defl_s *D) { return (float *)(D->vexp + D->k); }
+static float *space_lost2(const dtr_defl_s *D) { return (float *)(D->vexp + 2 * (size_t)D->k); }
+int defl_oz_setup(const dtr_defl_s *D, void *scratch, int *bad, cudaStream_t st) {
   const int k = D->k;
   const int64_t N = D->lat.N;
+  unsigned long long *sq = (unsigned long long *)scratch;
+  int *lost = (int *)(sq + k);
   DTR_CUDA(cudaMemsetAsync(D->vexp, 0, k * sizeof(int), st));
+  DTR_CUDA(cudaMemsetAsync(scratch, 0, k * (sizeof(*sq) + sizeof(int)), st));
   const unsigned grid = (unsigned)(8 * device_sms());
   // (an FP32 entry is exact down to 2^-31 of its column's largest; with an exponent of at least -60 subnormals are below)
   if (D->prec == DTR_F64) {
     k_oz_exp<double2><<<grid, 256, 0, st>>>((const double2 *)D->V, N, k, D->vexp, nullptr);
     k_oz_exp_finish<<<1, 256, 0, st>>>(D->vexp, k, 1023, 0x7ff, -800, bad);
-  } else {
-    if (D->prec == DTR_F32)
-      k_oz_exp<float2><<<grid, 256, 0, st>>>((const float2 *)D->V, N, k, D->vexp, nullptr);
-    else
-      k_oz_exp<bfc2><<<grid, 256, 0, st>>>((const bfc2 *)D->V, N, k, D->vexp, nullptr);
+    k_oz_squares<double2><<<grid, 256, 0, st>>>((const double2 *)D->V, N, k, D->vexp, sq, lost);
+  } else if (D->prec == DTR_F32) {
+    k_oz_exp<float2><<<grid, 256, 0, st>>>((const float2 *)D->V, N, k, D->vexp, nullptr);
     k_oz_exp_finish<<<1, 256, 0, st>>>(D->vexp, k, 127, 0xff, -60, bad);
+    k_oz_squares<float2><<<grid, 256, 0, st>>>((const float2 *)D->V, N, k, D->vexp, sq, lost);
+  } else {
+    k_oz_exp<bfc2><<<grid, 256, 0, st>>>((const bfc2 *)D->V, N, k, D->vexp, nullptr);
+    k_oz_exp_finish<<<1, 256, 0, st>>>(D->vexp, k, 127, 0xff, -60, bad);
+    k_oz_squares<bfc2><<<grid, 256, 0, st>>>((const bfc2 *)D->V, N, k, D->vexp, sq, lost);
   }
-  count_launches(2);
+  k_oz_limits<<<(unsigned)((k + 255) / 256), 256, 0, st>>>(sq, lost, k, D->prec == DTR_F64, space_v2(D), space_lost2(D),
+                                                           bad + 1);
+  count_launches(4);
   return DTR_OK;
 }
 
 // scratch in ints: [kBadC] and [kBadX], one pair of flags (the second found while the digits run) that send the
 // contraction or the expansion to the FP64 kernel; [kNeed] the sampled mass fell short, [kArrived] two block counters,
-// [kEz] exponents of Z's columns, [kCount] their nonzero entries, [kEw] exponents of the weights' columns, [kMass] masses
-// (64 bits, k b), behind them the weights' digit planes
-constexpr int kBadC = 0, kBadX = 2, kNeed = 4, kArrived = 5, kEz = 64, kCount = 128, kEw = 192, kMass = 256;
+// [kEz] exponents of Z's columns, [kCount] their nonzero entries, [kZ2] (in the contraction) their sums of squares, [kEw]
+// (in the expansion, in the same place) exponents of the weights' columns, [kLeast] (in
+// the expansion, which does not need the counts) least squares of x0's columns, [kMass] masses (64 bits, k b), behind them
+// the weights' digit planes
+constexpr int kBadC = 0, kBadX = 2, kNeed = 4, kArrived = 5, kEz = 64, kCount = 128, kLeast = 128, kZ2 = 192, kEw = 192, kMass = 256;
 static size_t planes_at(int k, int b) { return kMass + (size_t)2 * k * b; }
 size_t defl_oz_scratch_bytes(int k, int b) {
   return (planes_at(k, b) + (size_t)kDig * 2 * k * b) * sizeof(int);
@@ -583,12 +702,13 @@ template <typename VC> static int mass_t(const dtr_defl_s *D, const double2 *Z, 
   };
   unsigned long long *mass = (unsigned long long *)(sc + kMass);
   k_oz_mass<VC, false><<<grid((V + step - 1) / step), 256, 0, st>>>(
-      (const VC *)D->V, D->vexp, Z, sc + kEz, sc + kCount, sc + kBadC, sc + kNeed, k, b, V, step, mass,
-      (unsigned *)sc + kArrived, sc + (step > 1 ? kNeed : kBadC));
+      (const VC *)D->V, D->vexp, Z, sc + kEz, sc + kCount, sc + kBadC, sc + kNeed, k, b, V, step, space_v2(D),
+      space_lost2(D), mass, (unsigned *)sc + kZ2, (unsigned *)sc + kArrived, sc + (step > 1 ? kNeed : kBadC));
   count_launches(1);
   if (step > 1) {
     k_oz_mass<VC, true><<<grid(V - V / step), 256, 0, st>>>((const VC *)D->V, D->vexp, Z, sc + kEz, sc + kCount, sc + kBadC,
-                                                            sc + kNeed, k, b, V, step, mass, (unsigned *)sc + kArrived + 1,
+                                                            sc + kNeed, k, b, V, step, space_v2(D), space_lost2(D), mass,
+                                                            (unsigned *)sc + kZ2, (unsigned *)sc + kArrived + 1,
                                                             sc + kBadC);
     count_launches(1);
   }
@@ -625,30 +745,31 @@ int defl_oz_contract(const dtr_defl_s *D, const double2 *Z, int b, void *scratch
   return contract_t<bfc2>(D, Z, b, sc, nch, partial, st);
 }
 
-template <typename VC>
+template <typename VC, bool LOSSY>
 static int expand_t(const dtr_defl_s *D, int b, int *sc, double2 *x, cudaStream_t st) {
-  int rc = allow_smem(k_oz_expand<VC>, kXBytes);
+  int rc = allow_smem(k_oz_expand<VC, LOSSY>, kXBytes);
   if (rc) return rc;
   const int64_t N = D->lat.N, tiles = (N + kXD - 1) / kXD;
   const int nj = (b + kOJ - 1) / kOJ;
   int64_t gx = 2 * device_sms() / nj;
   if (gx < 1) gx = 1;
   if (gx > tiles) gx = tiles;
-  const float least = 16.f * (float)D->k * (D->prec == DTR_F64 ? 0x1p-13f : 0x1p-15f);
-  k_oz_expand<VC><<<dim3((unsigned)gx, nj), 256, kXBytes, st>>>((const VC *)D->V, D->vexp,
-                                                                 (const unsigned *)(sc + planes_at(D->k, b)), sc + kEw,
-                                                                 sc + kBadX, D->k, b, N, least, sc + kBadX + 1, x);
+  k_oz_expand<VC, LOSSY><<<dim3((unsigned)gx, nj), 256, kXBytes, st>>>(
+      (const VC *)D->V, D->vexp, (const unsigned *)(sc + planes_at(D->k, b)), sc + kEw, sc + kBadX, D->k, b, N,
+      (const float *)(sc + kLeast), sc + kBadX + 1, x);
   count_launches(1);
   return DTR_OK;
 }
 int defl_oz_expand(const dtr_defl_s *D, const double2 *W, int b, void *scratch, double2 *x, cudaStream_t st) {
   int *sc = (int *)scratch;
   DTR_CUDA(cudaMemsetAsync(sc + kBadX, 0, 2 * sizeof(int), st));
-  k_oz_weights<<<b, 256, 0, st>>>(W, D->vexp, D->k, b, (unsigned *)(sc + planes_at(D->k, b)), sc + kEw, sc + kBadX);
+  k_oz_weights<<<b, 256, 0, st>>>(W, D->vexp, D->k, b, D->prec == DTR_F64, (unsigned *)(sc + planes_at(D->k, b)),
+                                  sc + kEw, (float *)(sc + kLeast), sc + kBadX);
   count_launches(1);
-  if (D->prec == DTR_F64) return expand_t<double2>(D, b, sc, x, st);
-  if (D->prec == DTR_F32) return expand_t<float2>(D, b, sc, x, st);
-  return expand_t<bfc2>(D, b, sc, x, st);
+  if (D->prec == DTR_F64) return expand_t<double2, false>(D, b, sc, x, st);
+  if (D->prec == DTR_F32)
+    return D->vlossy ? expand_t<float2, true>(D, b, sc, x, st) : expand_t<float2, false>(D, b, sc, x, st);
+  return D->vlossy ? expand_t<bfc2, true>(D, b, sc, x, st) : expand_t<bfc2, false>(D, b, sc, x, st);
 }
 
 }  // namespace dtr

@@ -5,9 +5,10 @@
 
 namespace dtr {
 
-// Queues the exponents of V's columns into D->vexp (k ints, device); *bad (device): some column cannot be written in
-// integers.
-int defl_oz_setup(const dtr_defl_s *D, int *bad, cudaStream_t st);
+// Queues what the digits need of V into D->vexp (defl_oz_space_bytes(k) bytes, device); scratch: 12 k bytes; bad[0] (device):
+// some column cannot be written in integers, bad[1]: some FP32 or BF16 entries have more bits than their column's integers.
+size_t defl_oz_space_bytes(int k);
+int defl_oz_setup(const dtr_defl_s *D, void *scratch, int *bad, cudaStream_t st);
 size_t defl_oz_scratch_bytes(int k, int b);
 // Partial sums as k_defl_partial's, over *chunks (<= max_chunks) chunks of sites.
 int defl_oz_contract(const dtr_defl_s *D, const double2 *Z, int b, void *scratch, int max_chunks, double2 *partial,

@@ -187,8 +187,9 @@ struct dtr_defl_s {
   dtr_prec prec;
   void *V;            // row-major [dof][k] complex, FP64 (double2) or FP32 (float2)
   double *inv_lambda; // device, k
-  int *vexp;          // device, k (behind inv_lambda): exponents of V's columns (deflate_oz.cu)
+  int *vexp;          // device (behind inv_lambda): exponents of V's columns and sums of their squares (deflate_oz.cu)
   bool vexp_ok;       // and whether all columns have one
+  bool vlossy;        // FP32 or BF16 entries that have more bits than their column's integers
   double td[2];
   double tdg[16][2];  // T_D of Gamma_n (Gamma-insertion traces), valid where tdg_ok bit n is set
   unsigned tdg_ok;
