@@ -78,13 +78,16 @@ __device__ __forceinline__ float2 scaled(double2 v, int e) {
   return f64_to_f32(make_double2(scalbn(v.x, -e), scalbn(v.y, -e)));
 }
 __device__ __forceinline__ float2 scaled(bfc2 v, int e) { return scaled(__bfloat1622float2(v), e); }
-// whether the integer of an FP32 (or BF16) entry loses bits
-__device__ __forceinline__ int loses_bits(float f, int e) {
-  const unsigned b = __float_as_uint(f) & 0x7fffffffu;
+// whether the integer of an FP32 (or BF16) entry loses bits; b: its bits without the sign
+__device__ __forceinline__ int loses_bits(unsigned b, int e) {
   const int x = (int)(b >> 23), sh = x - 150 + kIntBits - e;
   return sh < 0 && b != 0u && (x == 0 || sh <= -24 || (b & ((1u << -sh) - 1u)) != 0u);
 }
-__device__ __forceinline__ int loses_bits(float2 v, int e) { return loses_bits(v.x, e) + loses_bits(v.y, e); }
+__device__ __forceinline__ int loses_bits(float2 v, int e) {
+  const unsigned a = __float_as_uint(v.x) & 0x7fffffffu, b = __float_as_uint(v.y) & 0x7fffffffu;
+  if ((int)(min(a, b) >> 23) >= 150 - kIntBits + e) return 0;  // nearly always
+  return loses_bits(a, e) + loses_bits(b, e);
+}
 __device__ __forceinline__ int loses_bits(bfc2 v, int e) { return loses_bits(__bfloat1622float2(v), e); }
 __device__ __forceinline__ int loses_bits(double2, int) { return 0; }  // (nearly all do: not counted)
 
@@ -552,7 +555,7 @@ __global__ void __launch_bounds__(256) k_oz_weights(const double2 *__restrict__ 
 // x[dof][j] = sum_m V[dof][m] W[m][j]: a block takes 64 dofs x 16 columns, 32 vectors (64 rows of Wd) a stage.
 // *small is set where 16 dofs of a column have squares below the column's `least` in sum (in the weights' units), with an
 // allowance for the FP32 and BF16 entries of the tile that lose bits (2/3 2^-110 each, for weights of at most one unit).
-// LOSSY: the space has such entries; looked for in any case, they cost 2 % of a projection.
+// LOSSY: the space has such entries (Gaussian FP32 ones from about 10^8 entries on).
 constexpr int kXD = 64, kXM = 32;
 constexpr int kXAs = (2 * kXM + 8) * 2, kXBs = (2 * kOJ + 8) * 2;
 constexpr int kXAp = kXD * kXAs, kXBp = 2 * kXM * kXBs;
@@ -688,11 +691,11 @@ template <typename K> static int allow_smem(K kern, int bytes) {
   return DTR_OK;
 }
 
-// Mass test: on part of the sites first, where Gaussian columns pass with a factor of 4 or more (at 16^3 x 32, k = 64,
-// b = 16 a sixth of them), and on the rest if that falls short.
+// Mass test: on part of the sites first, where Gaussian columns pass with a factor of 5 (at 16^3 x 32 a sixth of them in an
+// FP64 space, whose entries are all rounded, and a twelfth else), and on the rest if that falls short.
 template <typename VC> static int mass_t(const dtr_defl_s *D, const double2 *Z, int b, int *sc, cudaStream_t st) {
   const int V = (int)D->lat.V, k = D->k;
-  int step = (int)(std::sqrt((double)D->lat.N) / 200.0);
+  int step = (int)(std::sqrt((double)D->lat.N) / (D->prec == DTR_F64 ? 200.0 : 100.0));
   step = step < 1 ? 1 : step > 64 ? 64 : step;
   const int tiles = ((k + kMM - 1) / kMM) * ((b + kMJ - 1) / kMJ);
   auto grid = [&](int sites) {
