@@ -14,15 +14,15 @@
 // entries that are both small for their columns loses digits.  Two tests on the device send such blocks to the FP64
 // kernels (a point source; vectors that decay from opposite ends):
 //   C   S = sum of the products of the entries' moduli, in units of the columns' powers of two, must reach a bound T
-//       (k_oz_mass).  The digits' error goes with the squares that meet a rounded partner: T^2 = 4 (sum |v|^2 + sum |z|^2 where
-//       v is rounded + 2^-13 n for the dropped pairs), or n / 2 for n nonzero entries of z if that is less.  At S = T it is
-//       0.06 2^-53 of sum |v| |z|; FP64 chains come to 0.02 to 0.3 (49152 dofs, 24 families of graded, localised, sparse
-//       and plain columns).  Gaussian columns reach 6 T (FP64) and 12 T (FP32) there, growing with sqrt(n).
+//       (k_oz_mass).  The digits' error goes with the squares that meet a rounded partner: T^2 = 4 (sum |v|^2 + sum |z|^2
+//       where v is rounded + 2^-13 n for the dropped pairs), or n / 2 for n nonzero entries of z if that is less.  At S = T
+//       it is 0.06 2^-53 of sum |v| |z|; FP64 chains come to 0.02 to 0.3 (49152 dofs, 24 families of graded, localised,
+//       sparse and plain columns).  Gaussian columns reach 6 T (FP64) and 12 T (FP32) there, growing with sqrt(n).
 //   x0  sixteen neighbouring entries of a column, together, must be 2^50 times the error that they can have: that of V's
 //       entries where V is FP64 (2^-55 / sqrt(3) of the columns' powers of two, times the weights), and the digit pairs that
-//       are dropped (k_oz_expand).  FP32 and BF16 entries are exact in 54 bits down to 2^-30 of the largest, so that only the
-//       latter counts.  Largest errors of 16 entries above the line 7e-16, FP64 sums 9e-16 (spaces of the eigensolver, 8^4 to
-//       16^3 x 32, k = 16 to 100); its spaces at 16^4, FP64, are partly below.
+//       are dropped (k_oz_expand).  FP32 and BF16 entries are exact in 54 bits down to 2^-30 of the largest, those below are
+//       counted tile by tile.  Largest errors of 16 entries above the line 7e-16, FP64 sums 9e-16 (spaces of the
+//       eigensolver, 8^4 to 16^3 x 32, k = 16 to 100); its spaces at 16^4, FP64, are partly below.
 //
 // Digits come from shifts and byte permutes on the integer pipe.  A digit plane of Z that is zero over a stage is
 // skipped: probing noise (entries 0, +-1, +-i) has one digit.
@@ -319,11 +319,11 @@ __device__ __forceinline__ unsigned mag(double2 v, int e) {
 __device__ __forceinline__ unsigned mag(bfc2 v, int e) { return mag(__bfloat1622float2(v), e); }
 
 // mass[m b + j] += 2^16 sum over sites of |v| |z| (moduli as above: a lower bound, so part of the sites may do), z2[j] +=
-// sum |z|^2 (an upper bound); the last block compares with T and sets *fail for a pair that falls short.  Sites: every step-th (REST = false: here z
-// still holds k_oz_exp's fields, which the last block turns into exponents, setting *bad), or all but these (run if *need
-// is set).  A block: 64 vectors x 16 columns, stages of 4 sites as BF16 in shared memory; eight warps of 16 x 8 sums.  Its
-// loads are issued together, past the ends too (on valid entries, not used): one by one behind their tests a stage took
-// 8 us instead of 2.
+// sum |z|^2 (an upper bound); the last block compares with T and sets *fail for a pair that falls short.  Sites: every
+// step-th (REST = false: here ez still holds k_oz_exp's fields, which the last block turns into exponents, setting *bad),
+// or all but these (run if *need is set).  A block: 64 vectors x 16 columns, stages of 4 sites as BF16 in shared memory;
+// eight warps of 16 x 8 sums.  Its loads are issued together, past the ends too (on valid entries, not used): one by one
+// behind their tests a stage took 8 us instead of 2.
 constexpr int kMM = 64, kMJ = 16, kMK = 48;
 constexpr int kMAs = (kMM + 8) * 2, kMBs = (kMJ + 8) * 2;  // bytes of a dof row
 template <typename VC, bool REST>
@@ -675,9 +675,8 @@ int defl_oz_setup(const dtr_defl_s *D, void *scratch, int *bad, cudaStream_t st)
 // scratch in ints: [kBadC] and [kBadX], one pair of flags (the second found while the digits run) that send the
 // contraction or the expansion to the FP64 kernel; [kNeed] the sampled mass fell short, [kArrived] two block counters,
 // [kEz] exponents of Z's columns, [kCount] their nonzero entries, [kZ2] (in the contraction) their sums of squares, [kEw]
-// (in the expansion, in the same place) exponents of the weights' columns, [kLeast] (in
-// the expansion, which does not need the counts) least squares of x0's columns, [kMass] masses (64 bits, k b), behind them
-// the weights' digit planes
+// (in the expansion, in the same place) exponents of the weights' columns, [kLeast] (in the expansion, in the counts' place)
+// least squares of x0's columns, [kMass] masses (64 bits, k b), behind them the weights' digit planes
 constexpr int kBadC = 0, kBadX = 2, kNeed = 4, kArrived = 5, kEz = 64, kCount = 128, kLeast = 128, kZ2 = 192, kEw = 192, kMass = 256;
 static size_t planes_at(int k, int b) { return kMass + (size_t)2 * k * b; }
 size_t defl_oz_scratch_bytes(int k, int b) {
